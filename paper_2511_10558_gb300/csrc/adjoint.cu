@@ -133,11 +133,11 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const GradArgs a) {
   double* Jv = ws + 3 * R;     // [nnzJ]
   double* dT = Jv + n.nnzJ;    // [R]
   for (;;) {
-    if (threadIdx.x == 0) s_cell = atomicAdd(a.counter, 1);
+    if (threadIdx.x == 0) s_cell = next_cell(a.counter, a.order, a.C);
     __syncthreads();
     const int cell = s_cell;
     __syncthreads();
-    if (cell >= a.C) break;
+    if (cell < 0) break;
     double* grow = a.gcell + (size_t)cell * R;
     for (int j = threadIdx.x; j < R; j += NT) grow[j] = 0.0;
     double gnH = 0.0, gT = 0.0;

@@ -282,7 +282,9 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   a.stats = stats;
   if (tape) a.tape = tape->dev;
   a.ws_stride = plan.ws_stride;
-  const size_t ws_bytes = (size_t)grid * a.ws_stride * sizeof(double) + 256;
+  // the cells' order follows the counter when some CTA takes a second cell
+  const bool ordered = C > grid;
+  const size_t ws_bytes = (size_t)grid * a.ws_stride * sizeof(double) + 256 + (ordered ? (size_t)C * sizeof(int) : 0);
   void* ws = nullptr;
   cudaError_t e = cudaMallocAsync(&ws, ws_bytes, st);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(workspace)");
@@ -296,6 +298,12 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
     }
   }
   e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
+  if (e == cudaSuccess && ordered) {
+    int* order = (int*)((char*)a.counter + 256);
+    a.order = order;
+    e = (cudaError_t)launch_order(OrderArgs{C, phi, track, K, t0, t_end, t_end_cell, h.photo_alpha, h.photo_gamma,
+                                            h.cr_alpha, nullptr, order}, stream);
+  }
   if (e == cudaSuccess)
     e = (cudaError_t)(rk ? launch_solver_rk(a, plan, grid, stream) : launch_solver(a, plan, grid, stream));
   cudaError_t e2 = cudaFreeAsync(ws, st);
@@ -556,12 +564,20 @@ int cbx_grad_env(cbx_tape* tape, const double* cot_x, void* stream, double* g_lo
   const size_t b_gcell = ((size_t)C * h.R * 8 + 255) & ~size_t(255);
   const size_t b_ws = (size_t)grid * a.ws_stride * 8;
   char* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, b_gcell + b_ws + 256, st);
+  cudaError_t e = cudaMallocAsync((void**)&buf, b_gcell + b_ws + 256 + (size_t)C * sizeof(int), st);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(adjoint workspace)");
   a.gcell = (double*)buf;
   a.ws = (double*)(buf + b_gcell);
   a.counter = (int*)(buf + b_gcell + b_ws);
   e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
+  if (e == cudaSuccess && C > grid) {
+    OrderArgs oa{};
+    oa.C = C;
+    oa.nops = a.tape.nops;
+    oa.order = (int*)((char*)a.counter + 256);
+    a.order = oa.order;
+    e = (cudaError_t)launch_order(oa, stream);
+  }
   if (e == cudaSuccess) e = (cudaError_t)launch_grad(a, grid, stream);
   if (e == cudaSuccess && g_logalpha) e = (cudaError_t)launch_reduce_cells(a.gcell, C, h.R, g_logalpha, stream);
   if (e == cudaSuccess && (g_lnzeta || g_lnG0 || g_AV))

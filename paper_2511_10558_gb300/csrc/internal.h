@@ -87,6 +87,8 @@ struct HostNet {
   std::vector<int> rj;
   std::vector<double> gbeta, ggamma;
   double albedo = 0.0;  // omega
+  // means over the photo and the cosmic-ray reactions (estimate of a cell's cost)
+  float photo_alpha = 0.0f, photo_gamma = 0.0f, cr_alpha = 0.0f;
 };
 
 // Returns "" on success, else an error message.
@@ -112,6 +114,7 @@ struct SolveArgs {
   double* ws;      // per-CTA workspace, ws_stride doubles per CTA
   long long ws_stride;
   int* counter;    // next-cell counter, zero before the launch
+  const int* order;  // [C] cells in the order they are taken, or null: 0 .. C-1
   int piv_ints;    // pivot-list ints staged in shared memory (set by launch_solver)
   const double* track;  // [C][K][6] (t, n_H, T, A_V, G0, zeta) knots, or null: phi is constant
   int K;
@@ -150,7 +153,23 @@ struct GradArgs {
   double* ws;                  // per-CTA workspace, ws_stride doubles per CTA
   long long ws_stride;
   int* counter;
+  const int* order;            // [C] as in SolveArgs, or null
 };
+
+// Order of a launch's cells by estimated cost (a solve: from its environment;
+// a reverse sweep: from the ops on its tape), the costly ones first.
+struct OrderArgs {
+  int C;
+  const cbx_cell_params* phi;  // [C], or null with a track
+  const double* track;         // [C][K][6] or null (its first knot counts)
+  int K;
+  double t0, t_end;
+  const double* t_end_cell;    // [C] or null
+  float photo_alpha, photo_gamma, cr_alpha;
+  const int* nops;             // [C]: reverse sweep, or null
+  int* order;                  // [C] out
+};
+int launch_order(const OrderArgs& a, void* stream);
 
 // Adjoint launch: workspace doubles per CTA, CTAs per SM, launch.
 long long grad_workspace_doubles(int S, int R, int nnzJ);

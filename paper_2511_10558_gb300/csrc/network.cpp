@@ -148,6 +148,22 @@ std::string compile_network(const cbx_species* sp, int S, const cbx_reaction* rx
       }
   }
   n.tptr[kNumTypes] = (int)n.rj.size();
+  {
+    double pa = 0.0, pg = 0.0, ca = 0.0;
+    int np = 0, nc = 0;
+    for (int j = 0; j < R; ++j) {
+      if (n.rtype[j] == CBX_PHOTO) {
+        pa += n.alpha[j];
+        pg += n.gamma[j];
+        ++np;
+      } else if (n.rtype[j] == CBX_COSMIC_RAY || n.rtype[j] == CBX_CR_PHOTO) {
+        ca += n.rtype[j] == CBX_COSMIC_RAY ? n.alpha[j] : n.alpha[j] * n.gamma[j];
+        ++nc;
+      }
+    }
+    if (np) n.photo_alpha = (float)(pa / np), n.photo_gamma = (float)(pg / np);
+    if (nc) n.cr_alpha = (float)(ca / nc);
+  }
   // right-hand side gather lists, segmented
   n.spec_seg.push_back(0);
   n.seg_ptr.push_back(0);

@@ -156,6 +156,14 @@ extern "C" int cbx_solve_noalloc(cbx_network* net, const cbx_cell_params* phi, c
   a.ws = (double*)((unsigned char*)scratch + kCounterBytes);
   e = cudaMemsetAsync(a.counter, 0, sizeof(int), (cudaStream_t)stream);
   if (e != cudaSuccess) return fail(CBX_E_CUDA, std::string("cudaMemsetAsync(counter): ") + cudaGetErrorString(e));
+  const size_t used = kCounterBytes + (size_t)grid * stride * sizeof(double);
+  if (C > grid && (size_t)C * sizeof(int) <= kScratchBytes - used) {
+    int* order = (int*)((unsigned char*)scratch + used);
+    a.order = order;
+    e = (cudaError_t)cbx::launch_order(OrderArgs{C, phi, nullptr, 0, t0, t_end, nullptr, h.photo_alpha, h.photo_gamma,
+                                                 h.cr_alpha, nullptr, order}, stream);
+    if (e != cudaSuccess) return fail(CBX_E_CUDA, std::string("cell order launch: ") + cudaGetErrorString(e));
+  }
   e = (cudaError_t)launch_solver(a, plan, grid, stream);
   if (e != cudaSuccess) return fail(CBX_E_CUDA, std::string("solver launch: ") + cudaGetErrorString(e));
   return CBX_OK;

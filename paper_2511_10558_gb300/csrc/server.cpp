@@ -121,9 +121,10 @@ void size_request(ServerRequest* r, int max_ctas) {
 }
 
 // Device bytes of a launch of C cells of r's kind: inputs, outputs, end times,
-// status, workspace (pure arithmetic: safe under the lock).
+// status, workspace, order of the cells (pure arithmetic: safe under the lock).
 size_t launch_bytes(const ServerRequest* r, int C) {
-  return (size_t)C * r->cell_bytes + (size_t)std::min(C, r->grid_cap) * r->cta_bytes + 8192;
+  return (size_t)C * r->cell_bytes + (size_t)std::min(C, r->grid_cap) * r->cta_bytes +
+         (C > r->grid_cap ? (size_t)C * sizeof(int) : 0) + 8192;
 }
 
 bool same_kind(const ServerRequest* a, const ServerRequest* b) {

@@ -64,6 +64,12 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   return t;
 }
 
+// The next cell of the launch for this CTA, -1 when none is left.
+__device__ __forceinline__ int next_cell(int* counter, const int* order, int C) {
+  const int k = atomicAdd(counter, 1);
+  return k >= C ? -1 : (order ? order[k] : k);
+}
+
 // Deterministic block sum: warp trees, then the NW partials in a fixed order.
 // Every thread returns the same value. Contains two barriers.
 __device__ __forceinline__ double block_sum(double v, double* red) {
@@ -1954,11 +1960,11 @@ __global__ void __launch_bounds__(NT, 1) solve_kernel(const SolveArgs a) {
   }
   double* ws = a.ws + (size_t)blockIdx.x * a.ws_stride;
   for (;;) {
-    if (threadIdx.x == 0) s_cell = atomicAdd(a.counter, 1);
+    if (threadIdx.x == 0) s_cell = next_cell(a.counter, a.order, a.C);
     __syncthreads();
     const int cell = s_cell;
     __syncthreads();
-    if (cell >= a.C) break;
+    if (cell < 0) break;
     if constexpr (RK)
       solve_cell_rk<LT, GM>(a, cell, s, ws);
     else
