@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const GradArgs a) {
   double* Jv = ws + 3 * R;     // [nnzJ]
   double* dT = Jv + n.nnzJ;    // [R]
   for (;;) {
-    if (threadIdx.x == 0) s_cell = next_cell(a.counter, a.order, a.C);
+    if (tid() == 0) s_cell = next_cell(a.counter, a.order, a.C);
     __syncthreads();
     const int cell = s_cell;
     __syncthreads();
@@ -219,13 +219,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const GradArgs a) {
           grad_accumulate(n, kap, dT, s.y, g, c, grow, s.red, &gnH, &gT);
         } else if (kind == kOpRescale) {
           // Lam[1..q] <- T(rho)^T Lam[1..q]
-          if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-            if (lane < q * q) {
-              const int k = lane / q + 1, j = lane % q + 1;
-              s.Tm[(k - 1) * kMaxOrder + (j - 1)] = rescale_entry(k, j, v);
-            }
-          }
+          if (threadIdx.x < 32) rescale_matrix(q, v, s.Tm, s.red);
           __syncthreads();
           for (int i = threadIdx.x; i < S; i += NT) {
             double old[kMaxOrder];

@@ -40,23 +40,50 @@
 
 #include <cmath>
 #include <cstdio>
+#include <type_traits>
 
 #include "internal.h"
 
+// Threads of a CTA (one cell), CTAs per SM that the register budget is cut for,
+// and the most species the FP64 shared-memory LU takes (column groups per lane).
 #ifndef CBX_THREADS
 #define CBX_THREADS 256
+#endif
+#ifndef CBX_CTAS
+#define CBX_CTAS 1
+#endif
+#ifndef CBX_MAX_S
+#define CBX_MAX_S 256
+#endif
+// The lean shared-memory layout (see layout())
+#ifndef CBX_LEAN
+#define CBX_LEAN 0
 #endif
 
 namespace cbx {
 namespace {
 
-constexpr int NT = CBX_THREADS;  // threads per CTA
+constexpr int NT = CBX_THREADS;  // threads per CTA (one cell at a time)
 constexpr int NW = NT / 32;
+static_assert(NT == 32 || NT == 64 || NT == 128 || NT == 256, "a cell's threads");
 constexpr int kNewtonMaxIter = 4;
-constexpr int kMaxColRegs = 8;  // columns per lane in the LU update: S <= 256
+constexpr int kMaxColRegs = CBX_MAX_S / 32;  // column groups per lane in the LU update
 constexpr unsigned FULL = 0xffffffffu;
 
 // ---------------------------------------------------------------- helpers
+
+__device__ __forceinline__ int tid() { return threadIdx.x; }
+
+// Barrier among the threads of a cell.
+__device__ __forceinline__ void csync() {
+  if constexpr (NT == 32) __syncwarp();
+  else __syncthreads();
+}
+
+__device__ __forceinline__ int csync_or(int p) {
+  if constexpr (NT == 32) return __any_sync(FULL, p);
+  else return __syncthreads_or(p);
+}
 
 __device__ __forceinline__ unsigned long long globaltimer() {
   unsigned long long t;
@@ -70,44 +97,102 @@ __device__ __forceinline__ int next_cell(int* counter, const int* order, int C) 
   return k >= C ? -1 : (order ? order[k] : k);
 }
 
-// Deterministic block sum: warp trees, then the NW partials in a fixed order.
-// Every thread returns the same value. Contains two barriers.
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double s = 0.0;
-    for (int i = 0; i < NW; ++i) s += red[i];
-    if (threadIdx.x == 0) red[NW] = s;
+// ---- norms and other scalars
+//
+// A weighted sum of squares is reduced in a fixed order whatever NT: element i
+// belongs to chunk (i / 32) % 8, a chunk's 32 lanes are summed by a shuffle
+// tree, and the chunks are added in ascending order (chunks without elements
+// hold +0, which changes no sum of squares, and are left out). Warp 0 adds the
+// chunks and does what follows from the sum (the division and root, the rate
+// test, a power) alone: an FP64 instruction holds its sub-partition's pipe for
+// 64 cycles for each warp that issues it, and a division or root is a dozen of
+// them, so eight warps computing the same scalars hold it for thousands of cycles. Results go through `red`, in the half that the previous reduction
+// did not use, so that no barrier has to protect its readers.
+constexpr int kChunks = 8;
+
+// Partial sums of (a v_i w_i)^2 into slot[0..7]; no barrier.
+template <typename F>
+__device__ __forceinline__ void chunk_sums(F term, int S, double* slot) {
+  const int warp = tid() >> 5, lane = tid() & 31;
+  if constexpr (NT == 32 * kChunks) {
+    double acc = 0.0;
+    for (int i = tid(); i < S; i += NT) {
+      const double t = term(i);
+      acc = fma(t, t, acc);
+    }
+    if (32 * warp >= S) return;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    if (lane == 0) slot[warp] = acc;
+  } else {  // S <= 256 (the launch plan's rule)
+    for (int b = warp; 32 * b < S; b += NW) {
+      const int i = 32 * b + lane;
+      double acc = 0.0;
+      if (i < S) {
+        const double t = term(i);
+        acc = fma(t, t, acc);
+      }
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+      if (lane == 0) slot[b] = acc;
+    }
   }
-  __syncthreads();
-  const double s = red[NW];
-  __syncthreads();
+}
+
+__device__ __forceinline__ double chunk_total(const double* slot, int S) {
+  const int nb = min(kChunks, (S + 31) / 32);
+  double s = 0.0;
+  for (int b = 0; b < nb; ++b) s += slot[b];
   return s;
 }
 
-// sqrt(mean((a * v_i * w_i)^2)), w = reciprocal weights
-__device__ double wrms(const double* v, const double* w, double a, int S, double* red) {
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < S; i += NT) {
-    const double t = a * v[i] * w[i];
-    acc = fma(t, t, acc);
+// Deterministic block sum of one value per thread (NT = 256): warp trees, then
+// the NW partials in a fixed order. Every thread returns the same value.
+__device__ __forceinline__ double block_sum(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+  if ((tid() & 31) == 0) red[tid() >> 5] = v;
+  csync();
+  if (tid() < 32) {
+    double s = 0.0;
+    for (int i = 0; i < NW; ++i) s += red[i];
+    if (tid() == 0) red[NW] = s;
   }
-  return sqrt(block_sum(acc, red) / S);
+  csync();
+  const double s = red[NW];
+  csync();
+  return s;
 }
 
-// One thread computes pow(x, y); everybody gets it.
-__device__ double uniform_pow(double x, double y, double* slot) {
-  if (threadIdx.x == 0) *slot = pow(x, y);
-  __syncthreads();
-  const double v = *slot;
-  __syncthreads();
-  return v;
+// Scratch of the reductions: two halves of 64 doubles used in turn.
+struct Scratch {
+  double* red;
+  int half;
+  __device__ __forceinline__ double* next() {
+    half ^= 64;
+    return red + half;
+  }
+};
+
+// sqrt(mean((a * v_i * w_i)^2)), w = reciprocal weights. Two barriers.
+__device__ double wrms(const double* v, const double* w, double a, int S, Scratch& sc) {
+  double* slot = sc.next();
+  chunk_sums([&](int i) { return a * v[i] * w[i]; }, S, slot);
+  csync();
+  if (tid() < 32) {
+    const double r = sqrt(chunk_total(slot, S) / S);
+    if (tid() == 0) slot[kChunks] = r;
+  }
+  csync();
+  return slot[kChunks];
 }
 
-__device__ __forceinline__ double growth(double err, int p, double* slot) {
-  return err == 0.0 ? INFINITY : uniform_pow(err, -1.0 / p, slot);
+// One warp computes pow(x, y); everybody gets it. One barrier.
+__device__ double uniform_pow(double x, double y, Scratch& sc) {
+  double* slot = sc.next();
+  if (tid() < 32) {
+    const double v = pow(x, y);
+    if (tid() == 0) *slot = v;
+  }
+  csync();
+  return *slot;
 }
 
 // ---------------------------------------------------------------- chemistry
@@ -122,21 +207,21 @@ __device__ void rate_coefficients(const DevNet& n, const double* __restrict__ al
                                   double* kap) {
   const double lnT = log(p.T / 300.0);
   const double invT = 1.0 / p.T;
-  for (int e = n.tptr[CBX_TWO_BODY] + threadIdx.x; e < n.tptr[CBX_TWO_BODY + 1]; e += NT) {
+  for (int e = n.tptr[CBX_TWO_BODY] + tid(); e < n.tptr[CBX_TWO_BODY + 1]; e += NT) {
     const int j = __ldg(n.rj + e);
     kap[j] = alpha[j] * exp(__ldg(n.gbeta + e) * lnT - __ldg(n.ggamma + e) * invT) * p.n_H;
   }
-  for (int e = n.tptr[CBX_COSMIC_RAY] + threadIdx.x; e < n.tptr[CBX_COSMIC_RAY + 1]; e += NT) {
+  for (int e = n.tptr[CBX_COSMIC_RAY] + tid(); e < n.tptr[CBX_COSMIC_RAY + 1]; e += NT) {
     const int j = __ldg(n.rj + e);
     kap[j] = alpha[j] * p.zeta;
   }
-  for (int e = n.tptr[CBX_PHOTO] + threadIdx.x; e < n.tptr[CBX_PHOTO + 1]; e += NT) {
+  for (int e = n.tptr[CBX_PHOTO] + tid(); e < n.tptr[CBX_PHOTO + 1]; e += NT) {
     const int j = __ldg(n.rj + e);
     kap[j] = alpha[j] * p.G0 * exp(-__ldg(n.ggamma + e) * p.A_V);
   }
   // k = alpha (T/300)^beta E / (1 - omega) zeta, E in the gamma field
   const double crp = p.zeta * n.albedo_factor;
-  for (int e = n.tptr[CBX_CR_PHOTO] + threadIdx.x; e < n.tptr[CBX_CR_PHOTO + 1]; e += NT) {
+  for (int e = n.tptr[CBX_CR_PHOTO] + tid(); e < n.tptr[CBX_CR_PHOTO + 1]; e += NT) {
     const int j = __ldg(n.rj + e);
     kap[j] = alpha[j] * exp(__ldg(n.gbeta + e) * lnT) * __ldg(n.ggamma + e) * crp;
   }
@@ -150,7 +235,7 @@ __device__ void rate_coefficients(const DevNet& n, const double* __restrict__ al
 constexpr int kRatesPerPass = 8;
 __device__ void rhs(const DevNet& n, const double* __restrict__ kap, const double* y, double* f,
                     double* r, double* part) {
-  for (int j0 = threadIdx.x; j0 < n.R; j0 += kRatesPerPass * NT) {
+  for (int j0 = tid(); j0 < n.R; j0 += kRatesPerPass * NT) {
     int ia[kRatesPerPass], ib[kRatesPerPass];
     double kv[kRatesPerPass];
 #pragma unroll
@@ -171,8 +256,8 @@ __device__ void rhs(const DevNet& n, const double* __restrict__ kap, const doubl
       }
     }
   }
-  __syncthreads();
-  for (int sg = threadIdx.x; sg < n.nseg; sg += NT) {
+  csync();
+  for (int sg = tid(); sg < n.nseg; sg += NT) {
     const int e0 = __ldg(n.seg_ptr + sg), len = __ldg(n.seg_ptr + sg + 1) - e0;
     int t[kSegLen];
 #pragma unroll
@@ -188,21 +273,21 @@ __device__ void rhs(const DevNet& n, const double* __restrict__ kap, const doubl
     }
     part[sg] = acc0 + acc1;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n.S; i += NT) {
+  csync();
+  for (int i = tid(); i < n.S; i += NT) {
     double acc = 0.0;
     const int s1 = __ldg(n.spec_seg + i + 1);
     for (int sg = __ldg(n.spec_seg + i); sg < s1; ++sg) acc += part[sg];
     f[i] = acc;
   }
-  __syncthreads();
+  csync();
 }
 
 // Analytic Jacobian values per slot: J(i,l) = sum nu_ij dr_j/dx_l, with the
 // reaction partials g[2j+s] = d r_j / d x(reactant s).
 __device__ void jacobian(const DevNet& n, const double* __restrict__ kap, const double* y, double* g,
                          double* Jv) {
-  for (int j = threadIdx.x; j < n.R; j += NT) {
+  for (int j = tid(); j < n.R; j += NT) {
     const int b = n.rb[j];
     const double k = kap[j];
     if (b >= 0) {
@@ -213,10 +298,10 @@ __device__ void jacobian(const DevNet& n, const double* __restrict__ kap, const 
       g[2 * j + 1] = 0.0;
     }
   }
-  __syncthreads();
+  csync();
   // one warp per group of 32 slots; each lane sums its slot's terms in list
   // order (four loads ahead, one accumulator)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid() >> 5, lane = tid() & 31;
   for (int gi = warp; gi < n.njg; gi += NW) {
     const int s = __ldg(n.jg_slot + gi * 32 + lane);
     const int len = __ldg(n.jg_len + gi * 32 + lane);
@@ -242,7 +327,7 @@ __device__ void jacobian(const DevNet& n, const double* __restrict__ kap, const 
     }
     if (s >= 0) Jv[s] = acc;
   }
-  __syncthreads();
+  csync();
 }
 
 // ---------------------------------------------------------------- linear algebra
@@ -252,14 +337,14 @@ __host__ __device__ inline int lead_dim(int S) { return S | 1; }  // odd: confli
 template <typename LT>
 __device__ void build_matrix(const DevNet& n, const double* Jv, double c, LT* M) {
   const int S = n.S, ld = lead_dim(S);
-  for (int idx = threadIdx.x; idx < S * ld; idx += NT) M[idx] = LT(0);
-  __syncthreads();
-  for (int s = threadIdx.x; s < n.nnzJ; s += NT) {
+  for (int idx = tid(); idx < S * ld; idx += NT) M[idx] = LT(0);
+  csync();
+  for (int s = tid(); s < n.nnzJ; s += NT) {
     const int i = n.jrow[s], l = n.jcol[s];
     const double cj = c * Jv[s];
     M[i * ld + l] = (LT)(i == l ? 1.0 - cj : -cj);
   }
-  __syncthreads();
+  csync();
 }
 
 // ---------------------------------------------------------------- FP64 LU (Crout form)
@@ -273,7 +358,7 @@ __device__ void build_matrix(const DevNet& n, const double* Jv, double c, LT* M)
 // scaling) while the other warps work on their rows. Pivots k >= kd are
 // factored over the full ranges k+1..S-1 (entries outside the pattern are
 // exact zeros), without the per-pivot index lists, and there two pivots share
-// one barrier (dense_rank_rows).
+// one barrier (PairStep).
 
 // Index lists of the sparse pivots k < kd (from the network tables, or a
 // copy of their head in shared memory).
@@ -342,7 +427,7 @@ template <int MC>
 __device__ __forceinline__ void crout_rows(const PivLists& P, double* M, double* invd, int k, bool dense,
                                            int l0, int l1, int u0, int nu, bool next_in_l) {
   const int ld = lead_dim(P.S);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = tid() >> 5, lane = tid() & 31;
   int jc[MC];
   double uv[MC];
 #pragma unroll
@@ -375,11 +460,11 @@ __device__ __forceinline__ void crout_rows(const PivLists& P, double* M, double*
       __syncwarp();
       prep_pivot(P, M, invd, k + 1, lane);
     }
-    return;
+    if (NW > 1) return;
   }
   const int first = next_in_l ? l0 + 1 : l0;
-  const int nw = next_in_l ? NW - 1 : NW;
-  const int wi = next_in_l ? w - 1 : w;
+  const int nw = next_in_l && NW > 1 ? NW - 1 : NW;
+  const int wi = next_in_l && NW > 1 ? w - 1 : w;
   for (int e = first + wi; e < l1; e += 2 * nw) {
     const bool two = e + nw < l1;
     double* r0 = M + lrow(P, dense, k, e) * ld;
@@ -388,96 +473,64 @@ __device__ __forceinline__ void crout_rows(const PivLists& P, double* M, double*
   }
 }
 
-// Dense range, R pivots per barrier (R = 1 or 2): U rows k .. k+R-1 are final
-// on entry; every later row i takes their updates, all columns j >= k+R. For
-// R = 2 the L entry of column k+1 is formed first, b = M[i][k+1] - M[i][k]
-// U[k][k+1], then each element takes -M[i][k] U[k][j] and -b U[k+1][j] in
-// that order: the operations, and so the roundings, of two single-pivot
-// steps. Warp 0 takes rows p = k+R and p+1 and finishes both as U rows
-// (reciprocal pivot, pivot p applied to row p+1 from registers, scaling), so
-// that the next step finds them final; the other warps take the rows from
-// p+2 on, two at a time.
-#ifndef CBX_DENSE_PAIRS
-#define CBX_DENSE_PAIRS 1
-#endif
-
-template <int MC, int R>
-__device__ __forceinline__ void dense_rank_rows(double* M, double* invd, int S, int k) {
+// Dense range, first step: pivot k alone brings rows k+1 and k+2 to final (U
+// row k is final on entry). Warp 0 takes those two rows, finishes row k+1 as a
+// U row (reciprocal pivot, scaling), applies it to row k+2 from registers and
+// finishes that too; the other warps take the rows from k+3 on, two at a time.
+template <int MC>
+__device__ __forceinline__ void dense_first_rows(double* M, double* invd, int S, int k) {
   const int ld = lead_dim(S);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c0 = k + R, nu = S - c0;  // columns c0 .. S-1, lane + 32 m
-  double u0[MC], u1[MC];
+  const int w = tid() >> 5, lane = tid() & 31;
+  const int c0 = k + 1, nu = S - c0;  // columns c0 .. S-1, lane + 32 m
+  double u0[MC];
 #pragma unroll
-  for (int m = 0; m < MC; ++m) {
-    const bool in = lane + 32 * m < nu;
-    u0[m] = in ? M[k * ld + c0 + lane + 32 * m] : 0.0;
-    u1[m] = R == 2 && in ? M[(k + 1) * ld + c0 + lane + 32 * m] : 0.0;
-  }
-  const double u01 = R == 2 ? M[k * ld + k + 1] : 0.0;  // U(k, k+1)
-  // one row's update into x; returns its L entry of column k+1 (R = 2)
+  for (int m = 0; m < MC; ++m) u0[m] = lane + 32 * m < nu ? M[k * ld + c0 + lane + 32 * m] : 0.0;
   auto row_update = [&](const double* r, double (&x)[MC]) {
     const double a = r[k];
-    const double b = R == 2 ? fma(-a, u01, r[k + 1]) : 0.0;
 #pragma unroll
     for (int m = 0; m < MC; ++m) x[m] = lane + 32 * m < nu ? r[c0 + lane + 32 * m] : 0.0;
 #pragma unroll
     for (int m = 0; m < MC; ++m) x[m] = fma(-a, u0[m], x[m]);
-    if (R == 2) {
-#pragma unroll
-      for (int m = 0; m < MC; ++m) x[m] = fma(-b, u1[m], x[m]);
-    }
-    return b;
   };
   if (w == 0) {
     const int p = c0;
     double* rp = M + p * ld;
     double up[MC];  // row p: the diagonal at e = 0, U(p, :) after it
-    const double bp = row_update(rp, up);
+    row_update(rp, up);
     const double inv_p = __drcp_rn(__shfl_sync(FULL, up[0], 0));  // column p: lane 0, group 0
 #pragma unroll
     for (int m = 0; m < MC; ++m)
       if (lane + 32 * m >= 1) up[m] *= inv_p;
-    if (lane == 0) {
-      invd[p] = inv_p;
-      if (R == 2) rp[k + 1] = bp;
-    }
+    if (lane == 0) invd[p] = inv_p;
 #pragma unroll
     for (int m = 0; m < MC; ++m)
       if (lane + 32 * m < nu) rp[c0 + lane + 32 * m] = up[m];
     if (p + 1 < S) {
       double* rq = rp + ld;
       double xq[MC];
-      const double bq = row_update(rq, xq);
+      row_update(rq, xq);
       const double ap = __shfl_sync(FULL, xq[0], 0);  // L(p+1, p), stays
 #pragma unroll
       for (int m = 0; m < MC; ++m)
         if (lane + 32 * m >= 1) xq[m] = fma(-ap, up[m], xq[m]);
       const double inv_q = __drcp_rn(__shfl_sync(FULL, xq[0], 1));  // column p+1: lane 1, group 0
-      if (lane == 0) {
-        invd[p + 1] = inv_q;
-        if (R == 2) rq[k + 1] = bq;
-      }
+      if (lane == 0) invd[p + 1] = inv_q;
 #pragma unroll
       for (int m = 0; m < MC; ++m) {
         const int e = lane + 32 * m;
         if (e < nu) rq[c0 + e] = e <= 1 ? xq[m] : xq[m] * inv_q;
       }
     }
-    return;
+    if (NW > 1) return;
   }
-  const int first = c0 + 2, nrow = S - first, nw = NW - 1;
-  for (int e = w - 1; e < nrow; e += 2 * nw) {
+  const int first = c0 + 2, nrow = S - first, nw = NW > 1 ? NW - 1 : 1;
+  for (int e = NW > 1 ? w - 1 : 0; e < nrow; e += 2 * nw) {
     const bool two = e + nw < nrow;
     double* r0 = M + (first + e) * ld;
     double* r1 = two ? r0 + nw * ld : r0;
     double x0[MC], x1[MC];
-    const double b0 = row_update(r0, x0);
-    double b1 = 0.0;
-    if (two) b1 = row_update(r1, x1);
-    if (R == 2 && lane == 0) {
-      r0[k + 1] = b0;
-      if (two) r1[k + 1] = b1;
-    }
+    row_update(r0, x0);
+    if (two) row_update(r1, x1);
 #pragma unroll
     for (int m = 0; m < MC; ++m) {
       if (lane + 32 * m < nu) {
@@ -488,29 +541,211 @@ __device__ __forceinline__ void dense_rank_rows(double* M, double* invd, int S, 
   }
 }
 
+// Dense range, two pivots a step: U rows k and k+1 are final; every later row i
+// takes their updates. Lanes hold the columns from k+1 on (e = column - (k+1)):
+// the first pass, -M[i][k] U[k][j], leaves the row's L entry b of column k+1 in
+// lane 0, from where a shuffle gives it to the second pass, -b U[k+1][j]: the
+// operations, and so the roundings, of two single-pivot steps. (An FP64
+// instruction costs its sub-partition 64 cycles however few lanes need it, so
+// forming b by an instruction of its own would make it 2 MC + 1 a row instead
+// of 2 MC.)
+template <int MC>
+struct PairStep {
+  int k, ld, lane, nu;
+  double u0[MC], u1[MC];
+
+  __device__ __forceinline__ PairStep(const double* M, int S, int k_, int lane_)
+      : k(k_), ld(lead_dim(S)), lane(lane_), nu(S - k_ - 1) {
+#pragma unroll
+    for (int m = 0; m < MC; ++m) {
+      const bool in = lane + 32 * m < nu;
+      u0[m] = in ? M[k * ld + k + 1 + lane + 32 * m] : 0.0;
+      u1[m] = in ? M[(k + 1) * ld + k + 1 + lane + 32 * m] : 0.0;
+    }
+  }
+
+  __device__ __forceinline__ void load(const double* r, double& a, double (&x)[MC]) const {
+    a = r[k];
+#pragma unroll
+    for (int m = 0; m < MC; ++m) x[m] = lane + 32 * m < nu ? r[k + 1 + lane + 32 * m] : 0.0;
+  }
+
+  __device__ __forceinline__ void update(double a, double (&x)[MC]) const {
+#pragma unroll
+    for (int m = 0; m < MC; ++m) x[m] = fma(-a, u0[m], x[m]);
+    const double b = __shfl_sync(FULL, x[0], 0);
+#pragma unroll
+    for (int m = 0; m < MC; ++m)
+      if (m > 0 || lane > 0) x[m] = fma(-b, u1[m], x[m]);
+  }
+
+  __device__ __forceinline__ void store(double* r, const double (&x)[MC]) const {
+#pragma unroll
+    for (int m = 0; m < MC; ++m)
+      if (lane + 32 * m < nu) r[k + 1 + lane + 32 * m] = x[m];
+  }
+
+  // Rows p = k+2 and p+1 to final U rows (warp 0): their updates, reciprocal
+  // pivot p, pivot p applied to row p+1 from registers, reciprocal pivot p+1.
+  __device__ __forceinline__ void finish_rows(double* M, double* invd, int S) const {
+    const int p = k + 2;
+    double* rp = M + p * ld;
+    double up[MC], xq[MC], a;
+    load(rp, a, up);
+    update(a, up);
+    const double inv_p = __drcp_rn(__shfl_sync(FULL, up[0], 1));
+#pragma unroll
+    for (int m = 0; m < MC; ++m)
+      if (lane + 32 * m >= 2) up[m] *= inv_p;
+    if (lane == 0) invd[p] = inv_p;
+    store(rp, up);
+    if (p + 1 < S) {
+      load(rp + ld, a, xq);
+      update(a, xq);
+      const double ap = __shfl_sync(FULL, xq[0], 1);  // L(p+1, p), stays
+#pragma unroll
+      for (int m = 0; m < MC; ++m)
+        if (lane + 32 * m >= 2) xq[m] = fma(-ap, up[m], xq[m]);
+      const double inv_q = __drcp_rn(__shfl_sync(FULL, xq[0], 2));
+      if (lane == 0) invd[p + 1] = inv_q;
+#pragma unroll
+      for (int m = 0; m < MC; ++m)
+        if (lane + 32 * m >= 3) xq[m] *= inv_q;
+      store(rp + ld, xq);
+    }
+  }
+};
+
+// The pair steps are a pipeline between warp 0, which finishes the next two U
+// rows, and the other warps (workers), which own the remaining rows (row i
+// belongs to worker i mod (NW - 1) in every step, so a row needs no barrier
+// between its updates). Two events replace the block barrier: "rows k+2, k+3
+// are U rows" (warp 0 to the workers) and "rows k+4, k+5 have the step's
+// updates" (workers to warp 0, sent as soon as each worker has done its first
+// rows, which are those). Warp 0 finishes the next rows while the workers are
+// still on the rest of theirs, and a worker goes on to the next step without
+// waiting for the others' last rows. An event is a named barrier on which one
+// side arrives and the other waits: the first has one for each sub-partition
+// (workers w and w + 4 share it), and both are used in turn by even and odd
+// steps, because a side may be one step ahead of the other (never two: warp 0
+// finishes step s+1 after every worker's first rows of step s, a worker begins
+// step s+2 after that). One cell alone, cycles a factorisation: 150 species 652k
+// -> 585k (470k of them here; its 25.2k FP64 warp instructions take 403k at one
+// per 16 cycles), 97 species 237k -> 214k, 61 species 95k -> 87k.
+//
+// The barrier numbers are immediates: a number in a register would make the
+// kernel claim all sixteen, which limits the CTAs on an SM.
+template <int ID, int N>
+__device__ __forceinline__ void bar_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
+template <int ID, int N>
+__device__ __forceinline__ void bar_wait() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
+
+// Workers on sub-partition G (warps w >= 1 with w % 4 = G).
+template <int G>
+constexpr int kGroupWorkers = (NW + 3 - G) / 4 - (G == 0);
+
+template <int G, bool WAIT>
+__device__ __forceinline__ void urows_event(int step) {
+  constexpr int n = 32 + 32 * kGroupWorkers<G>;
+  if constexpr (n > 32) {
+    if (step & 1) {
+      if constexpr (WAIT) bar_wait<3 + 2 * G + 1, n>();
+      else bar_arrive<3 + 2 * G + 1, n>();
+    } else {
+      if constexpr (WAIT) bar_wait<3 + 2 * G, n>();
+      else bar_arrive<3 + 2 * G, n>();
+    }
+  }
+}
+
+// Warp 0: rows k+2, k+3 of this step are U rows.
+__device__ __forceinline__ void urows_send(int step) {
+  urows_event<0, false>(step);
+  urows_event<1, false>(step);
+  urows_event<2, false>(step);
+  urows_event<3, false>(step);
+}
+
+__device__ __forceinline__ void urows_wait(int step, int w) {
+  switch (w & 3) {
+    case 0: urows_event<0, true>(step); break;
+    case 1: urows_event<1, true>(step); break;
+    case 2: urows_event<2, true>(step); break;
+    default: urows_event<3, true>(step); break;
+  }
+}
+
+// A worker has done its first rows of this step.
+__device__ __forceinline__ void first_send(int step) {
+  if constexpr (NW > 1) {
+    if (step & 1) bar_arrive<2, NT>();
+    else bar_arrive<1, NT>();
+  }
+}
+
+__device__ __forceinline__ void first_wait(int step) {
+  if constexpr (NW > 1) {
+    if (step & 1) bar_wait<2, NT>();
+    else bar_wait<1, NT>();
+  }
+}
+
+// One step of the workers (every warp but warp 0).
+template <int MC>
+__device__ __forceinline__ void pair_rows(double* M, int S, int k, int step, int w, int lane) {
+  constexpr int nw = NW > 1 ? NW - 1 : 1;
+  const int ld = lead_dim(S), first = k + 4;
+  const PairStep<MC> st(M, S, k, lane);
+  bool sent = false;
+  for (int i = first + ((w - 1) + nw * S - first) % nw; i < S; i += 2 * nw) {
+    const bool two = i + nw < S;
+    double* r0 = M + i * ld;
+    double* r1 = two ? r0 + nw * ld : r0;
+    double x0[MC], x1[MC], a0, a1;
+    st.load(r0, a0, x0);
+    st.load(r1, a1, x1);
+    st.update(a0, x0);
+    if (two) st.update(a1, x1);
+    st.store(r0, x0);
+    if (two) st.store(r1, x1);
+    if (!sent) {
+      first_send(step);
+      sent = true;
+    }
+  }
+  if (!sent) first_send(step);
+}
+
+template <int MC>
+__device__ __forceinline__ void pair_finish(double* M, double* invd, int S, int k, int lane) {
+  const PairStep<MC> st(M, S, k, lane);
+  st.finish_rows(M, invd, S);
+}
+
 // at most DENSE_PAIR_COLS columns (4 groups per lane): the step's register
 // footprint stays within the kernel's budget
 constexpr int DENSE_PAIR_COLS = 128;
 
-template <int R>
-__device__ __forceinline__ void dense_rank_step(double* M, double* invd, int S, int k) {
-  switch ((S - k - R + 31) >> 5) {
-    case 1: dense_rank_rows<1, R>(M, invd, S, k); break;
-    case 2: dense_rank_rows<2, R>(M, invd, S, k); break;
-    case 3: dense_rank_rows<3, R>(M, invd, S, k); break;
-    default: dense_rank_rows<4, R>(M, invd, S, k); break;
+// f<groups>(), groups = the column groups of 32 for nu columns (at most 4)
+template <typename F>
+__device__ __forceinline__ void by_groups(int nu, F f) {
+  switch ((nu + 31) >> 5) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: if constexpr (kMaxColRegs >= 2) f(std::integral_constant<int, 2>()); break;
+    case 3: if constexpr (kMaxColRegs >= 3) f(std::integral_constant<int, 3>()); break;
+    default: if constexpr (kMaxColRegs >= 4) f(std::integral_constant<int, 4>()); break;
   }
 }
 
 __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
   const int S = P.S, ld = lead_dim(S), kd = P.kd;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = tid() >> 5, lane = tid() & 31;
   if (w == 0) prep_pivot(P, M, invd, 0, lane);
-  __syncthreads();
+  csync();
   // with pairs, the single-pivot loop stops at kp: the first dense pivot
   // with at most DENSE_PAIR_COLS columns after it
   const int kp = max(kd, S - 1 - DENSE_PAIR_COLS);
-  const bool pairs = CBX_DENSE_PAIRS && S - kp >= 3;
+  const bool pairs = S - kp >= 3;
   const int k_single = pairs ? kp : S - 1;
   for (int k = 0; k < k_single; ++k) {
     const bool dense = k >= kd;
@@ -531,34 +766,47 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
     if (nu > 0) {
       switch ((nu + 31) >> 5) {
         case 1: crout_rows<1>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        case 2: crout_rows<2>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        case 3: crout_rows<3>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        case 4: crout_rows<4>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        case 5: crout_rows<5>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        case 6: crout_rows<6>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        case 7: crout_rows<7>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
-        default: crout_rows<8>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        case 2: if constexpr (kMaxColRegs >= 2) crout_rows<2>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        case 3: if constexpr (kMaxColRegs >= 3) crout_rows<3>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        case 4: if constexpr (kMaxColRegs >= 4) crout_rows<4>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        case 5: if constexpr (kMaxColRegs >= 5) crout_rows<5>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        case 6: if constexpr (kMaxColRegs >= 6) crout_rows<6>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        case 7: if constexpr (kMaxColRegs >= 7) crout_rows<7>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
+        default: if constexpr (kMaxColRegs >= 8) crout_rows<8>(P, M, invd, k, dense, l0, l1, u0, nu, next_in_l); break;
       }
     } else if (w == 0 && next_in_l) {
       prep_pivot(P, M, invd, k + 1, lane);
     }
-    __syncthreads();
+    csync();
   }
   if (pairs) {
     // U row kp is final; pivot kp alone brings rows kp+1 and kp+2 to final,
     // then pivots go in pairs while rows remain below them
-    dense_rank_step<1>(M, invd, S, kp);
-    __syncthreads();
-    for (int k = kp + 1; k + 2 < S; k += 2) {
-      dense_rank_step<2>(M, invd, S, k);
-      __syncthreads();
+    by_groups(S - kp - 1, [&](auto mc) { dense_first_rows<mc.value>(M, invd, S, kp); });
+    csync();
+    int step = 0;
+    for (int k = kp + 1; k + 2 < S; k += 2, ++step) {
+      if (w == 0) {
+        if (step > 0) first_wait(step - 1);
+        by_groups(S - k - 1, [&](auto mc) { pair_finish<mc.value>(M, invd, S, k, lane); });
+        urows_send(step);
+      }
+      if (w > 0 || NW == 1) {
+        if (step > 0) urows_wait(step - 1, w);
+        by_groups(S - k - 1, [&](auto mc) { pair_rows<mc.value>(M, S, k, step, w, lane); });
+      }
     }
+    if (step > 0) {  // the last step's events
+      if (w == 0) first_wait(step - 1);
+      else urows_wait(step - 1, w);
+    }
+    csync();
   }
   // L(:,k) /= pivot_k: M now holds L (unit lower), the pivots in invd (as
   // reciprocals) and U (unit upper), so both triangular solves are unit.
-  for (int i = 1 + (threadIdx.x >> 5); i < S; i += NW)
+  for (int i = 1 + (tid() >> 5); i < S; i += NW)
     for (int k = lane; k < i; k += 32) M[i * ld + k] *= invd[k];
-  __syncthreads();
+  csync();
 }
 
 // Triangular solves with the Crout factors, blocks of 32 with look-ahead.
@@ -574,10 +822,13 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
 // block is the chain plus an eighth of the next block's update.
 constexpr int LA_COLS = 8;
 
-// bulk-update worker index of warp w (0..5 for the warps not on warp 0's
-// sub-partition), or -1
-__device__ __forceinline__ int la_worker(int w) { return (w & 3) == 0 ? -1 : (w >> 2) * 3 + (w & 3) - 1; }
-constexpr int LA_WORKERS = (NW / 4) * 3;
+// bulk-update worker index of warp w (of eight warps the six not on warp 0's
+// sub-partition; of one the only one), or -1
+__device__ __forceinline__ int la_worker(int w) {
+  if (NW >= 4) return (w & 3) == 0 ? -1 : (w >> 2) * 3 + (w & 3) - 1;
+  return NW == 2 ? w - 1 : 0;
+}
+constexpr int LA_WORKERS = NW >= 4 ? (NW / 4) * 3 : 1;
 
 // v[i] -= sum_{c < nc} row_i[c] y[c] for rows i in [i0, i1), one thread per
 // row of this worker
@@ -599,27 +850,32 @@ __device__ __forceinline__ void la_bulk(const double* M, int ld, const double* y
 }
 
 // part[32 w + lane] = sum of row (r0 + lane)'s entries in columns
-// c0 + LA_COLS w .. (below c0 + nc) times y; warps 0..3
+// c0 + LA_COLS w .. (below c0 + nc) times y, for w = 0..3 (one a warp where
+// there are four)
 __device__ __forceinline__ void la_next(const double* M, int ld, const double* v, int c0, int nc, int r0, int r1,
-                                        double* part, int w, int lane) {
-  const int i = r0 + lane, cw = LA_COLS * w;
-  double p = 0.0, q = 0.0;
-  if (i < r1) {
-    const double* row = M + i * ld + c0 + cw;
-    const double* y = v + c0 + cw;
+                                        double* part, int warp, int lane) {
+  const int i = r0 + lane;
 #pragma unroll
-    for (int c = 0; c < LA_COLS; c += 2) {
-      if (cw + c < nc) p = fma(row[c], y[c], p);
-      if (cw + c + 1 < nc) q = fma(row[c + 1], y[c + 1], q);
+  for (int w = warp; w < 4; w += NW) {
+    const int cw = LA_COLS * w;
+    double p = 0.0, q = 0.0;
+    if (i < r1) {
+      const double* row = M + i * ld + c0 + cw;
+      const double* y = v + c0 + cw;
+#pragma unroll
+      for (int c = 0; c < LA_COLS; c += 2) {
+        if (cw + c < nc) p = fma(row[c], y[c], p);
+        if (cw + c + 1 < nc) q = fma(row[c + 1], y[c + 1], q);
+      }
     }
+    part[32 * w + lane] = p + q;
   }
-  part[32 * w + lane] = p + q;
 }
 
 // v <- D^{-1} L^{-1} v (L unit lower, D the pivots with reciprocals in invd);
 // D^{-1} last, element-wise. part: 128 doubles of shared scratch.
 __device__ void forward_crout64(const double* M, const double* invd, int S, double* v, double* part) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, ld = lead_dim(S);
+  const int w = tid() >> 5, lane = tid() & 31, ld = lead_dim(S);
   const int nblk = (S + 31) / 32, wk = la_worker(w);
   for (int b = 0; b < nblk; ++b) {
     const int kb = 32 * b, nb = min(32, S - kb);
@@ -630,31 +886,40 @@ __device__ void forward_crout64(const double* M, const double* invd, int S, doub
         if (b > 0) val -= (part[lane] + part[32 + lane]) + (part[64 + lane] + part[96 + lane]);
       }
       const double* row = M + (kb + min(lane, nb - 1)) * ld + kb;
+      if (nb == 32) {
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        if (c < nb) {
+        for (int c = 0; c < 31; ++c) {
           const double yc = __shfl_sync(FULL, val, c);
-          if (lane > c && lane < nb) val = fma(-row[c], yc, val);
+          if (lane > c) val = fma(-row[c], yc, val);
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < 31; ++c) {
+          if (c < nb - 1) {
+            const double yc = __shfl_sync(FULL, val, c);
+            if (lane > c && lane < nb) val = fma(-row[c], yc, val);
+          }
         }
       }
       if (lane < nb) v[kb + lane] = val;
-    } else if (wk >= 0 && b > 0) {
+    }
+    if (wk >= 0 && b > 0) {
       // block b-1 (full) on the rows below block b (block b took it through
       // the partial sums)
       la_bulk(M, ld, v + kb - 32, kb - 32, 32, v, kb + 32, S, wk, lane);
     }
-    __syncthreads();
+    csync();
     if (b + 1 < nblk && w < 4) la_next(M, ld, v, kb, 32, kb + 32, S, part, w, lane);
-    __syncthreads();
+    csync();
   }
-  for (int i = threadIdx.x; i < S; i += NT) v[i] *= invd[i];
-  __syncthreads();
+  for (int i = tid(); i < S; i += NT) v[i] *= invd[i];
+  csync();
 }
 
 // v <- U^{-1} v for the unit upper Crout factor, blocks of 32 from the bottom
 // (the bottom block may be partial; the others are full).
 __device__ void backward_crout64(const double* M, int S, double* v, double* part) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, ld = lead_dim(S);
+  const int w = tid() >> 5, lane = tid() & 31, ld = lead_dim(S);
   const int nblk = (S + 31) / 32, wk = la_worker(w);
   for (int b = nblk - 1; b >= 0; --b) {
     const int kb = 32 * b, nb = min(32, S - kb);
@@ -665,23 +930,32 @@ __device__ void backward_crout64(const double* M, int S, double* v, double* part
         if (b + 1 < nblk) val -= (part[lane] + part[32 + lane]) + (part[64 + lane] + part[96 + lane]);
       }
       const double* row = M + (kb + min(lane, nb - 1)) * ld + kb;
+      if (nb == 32) {
 #pragma unroll
-      for (int c = 31; c >= 0; --c) {
-        if (c < nb) {
+        for (int c = 31; c > 0; --c) {
           const double xc = __shfl_sync(FULL, val, c);
           if (lane < c) val = fma(-row[c], xc, val);
         }
+      } else {
+#pragma unroll
+        for (int c = 30; c > 0; --c) {
+          if (c < nb) {
+            const double xc = __shfl_sync(FULL, val, c);
+            if (lane < c) val = fma(-row[c], xc, val);
+          }
+        }
       }
       if (lane < nb) v[kb + lane] = val;
-    } else if (wk >= 0 && b + 1 < nblk && b > 0) {
+    }
+    if (wk >= 0 && b + 1 < nblk && b > 0) {
       // block b+1 (possibly the partial bottom block) on the rows above block b
       // (block b took it through the partial sums)
       const int kn = kb + 32;
       la_bulk(M, ld, v + kn, kn, min(32, S - kn), v, 0, kb, wk, lane);
     }
-    __syncthreads();
+    csync();
     if (b > 0 && w < 4) la_next(M, ld, v, kb, nb, kb - 32, kb, part, w, lane);
-    __syncthreads();
+    csync();
   }
 }
 
@@ -709,11 +983,11 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
 template <typename LT, bool FULL, int RPT>
 __device__ __forceinline__ void panel_factor(LT* M, LT* invd, int S, int ld, int kb, int nb) {
-  const int tid = threadIdx.x;
+  const int t = tid();
   LT r[RPT][NB];
 #pragma unroll
   for (int p = 0; p < RPT; ++p) {
-    const int i = kb + tid + NT * p;
+    const int i = kb + t + NT * p;
 #pragma unroll
     for (int jj = 0; jj < NB; ++jj) r[p][jj] = i < S && (FULL || jj < nb) ? M[i * ld + kb + jj] : LT(0);
   }
@@ -721,17 +995,17 @@ __device__ __forceinline__ void panel_factor(LT* M, LT* invd, int S, int ld, int
   for (int c = 0; c < NB; ++c) {
     if (FULL || c < nb) {
       const int k = kb + c;
-      if (tid == k - kb) {  // the pivot row is row kb + c, owned by thread c (p = 0)
+      if (t == k - kb) {  // the pivot row is row kb + c, owned by thread c (p = 0)
 #pragma unroll
         for (int jj = c; jj < NB; ++jj)
           if (FULL || jj < nb) M[k * ld + kb + jj] = r[0][jj];
       }
-      __syncthreads();
+      csync();
       const LT* prow = M + k * ld + kb;
       const LT inv = recip(prow[c]);
 #pragma unroll
       for (int p = 0; p < RPT; ++p) {
-        const int i = kb + tid + NT * p;
+        const int i = kb + t + NT * p;
         if (i < S && i > k) {
           const LT l = r[p][c] * inv;
           r[p][c] = l;
@@ -740,13 +1014,13 @@ __device__ __forceinline__ void panel_factor(LT* M, LT* invd, int S, int ld, int
             if (FULL || jj < nb) r[p][jj] -= l * prow[jj];
         }
       }
-      if (tid == 0) invd[k] = inv;
+      if (t == 0) invd[k] = inv;
     }
   }
-  __syncthreads();
+  csync();
 #pragma unroll
   for (int p = 0; p < RPT; ++p) {
-    const int i = kb + tid + NT * p;
+    const int i = kb + t + NT * p;
     if (i >= S) continue;
     if (i >= kb + nb) {
 #pragma unroll
@@ -759,7 +1033,7 @@ __device__ __forceinline__ void panel_factor(LT* M, LT* invd, int S, int ld, int
         if (kb + jj < i) M[i * ld + kb + jj] = r[p][jj];
     }
   }
-  __syncthreads();
+  csync();
 }
 
 // Forward substitution of one column (NB values in registers) with the unit
@@ -781,7 +1055,7 @@ __device__ __forceinline__ void panel_u12(LT* M, int S, int ld, int kb, int nb) 
   if (ncol + nb <= NT) {
     // one pass: threads < ncol take A12 columns, the next nb the identity
     // columns; L11^{-1} is written over L11 after everyone has read it
-    const int t = threadIdx.x;
+    const int t = tid();
     const bool a12 = t < ncol, ident = !a12 && t < ncol + nb;
     const int col = ke + t, jj = t - ncol;
     LT v[NB];
@@ -789,7 +1063,7 @@ __device__ __forceinline__ void panel_u12(LT* M, int S, int ld, int kb, int nb) 
     for (int r = 0; r < NB; ++r)
       v[r] = a12 && (FULL || r < nb) ? M[(kb + r) * ld + col] : (ident && r == jj ? LT(1) : LT(0));
     if (a12 || ident) l11_solve<LT, FULL>(L, ld, nb, v);
-    __syncthreads();
+    csync();
     if (a12) {
 #pragma unroll
       for (int r = 0; r < NB; ++r)
@@ -799,11 +1073,11 @@ __device__ __forceinline__ void panel_u12(LT* M, int S, int ld, int kb, int nb) 
       for (int r = 0; r < NB; ++r)
         if (r > jj && (FULL || r < nb)) M[(kb + r) * ld + kb + jj] = v[r];
     }
-    __syncthreads();
+    csync();
     return;
   }
   // U12 = L11^{-1} A12, one column per thread (A12 does not overlap L11)
-  for (int t = threadIdx.x; t < ncol; t += NT) {
+  for (int t = tid(); t < ncol; t += NT) {
     const int col = ke + t;
     LT v[NB];
 #pragma unroll
@@ -814,18 +1088,18 @@ __device__ __forceinline__ void panel_u12(LT* M, int S, int ld, int kb, int nb) 
       if (FULL || r < nb) M[(kb + r) * ld + col] = v[r];
   }
   // L11^{-1}: identity columns, written over L11 after everyone has read it
-  const int jj = threadIdx.x;
+  const int jj = tid();
   LT v[NB];
 #pragma unroll
   for (int r = 0; r < NB; ++r) v[r] = r == jj ? LT(1) : LT(0);
   if (jj < nb) l11_solve<LT, FULL>(L, ld, nb, v);
-  __syncthreads();
+  csync();
   if (jj < nb) {
 #pragma unroll
     for (int r = 0; r < NB; ++r)
       if (r > jj && (FULL || r < nb)) M[(kb + r) * ld + kb + jj] = v[r];
   }
-  __syncthreads();
+  csync();
 }
 
 // A22 -= L21 U12 over rows/cols [ke, S): warps take TR-row strips, lanes the
@@ -833,7 +1107,7 @@ __device__ __forceinline__ void panel_u12(LT* M, int S, int ld, int kb, int nb) 
 template <typename LT, int NG, int TR>
 __device__ __forceinline__ void trailing_update_ng(LT* M, int S, int ld, int kb, int nb) {
   const int ke = kb + nb, ncol = S - ke;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid() >> 5, lane = tid() & 31;
   bool colok[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) colok[g] = lane + 32 * g < ncol;
@@ -914,7 +1188,7 @@ template <int TN>
 __device__ __forceinline__ void tc_rect(float* M, int ld, int k0, int K, int r0, int r1, int c0, int c1) {
   const int m = r1 - r0, n = c1 - c0;
   if (m <= 0 || n <= 0) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int warp = tid() >> 5, lane = tid() & 31, g = lane >> 2, q = lane & 3;
   const int nbr = (m + 15) / 16, nbc = (n + 8 * TN - 1) / (8 * TN);
   for (int blk = warp; blk < nbr * nbc; blk += NW) {
     const int rt = r0 + (blk / nbc) * 16, ct = c0 + (blk % nbc) * 8 * TN;
@@ -978,22 +1252,22 @@ __device__ __forceinline__ void trailing_update(LT* M, int S, int ld, int kb, in
   // form below measured 2.5 % faster over a whole solve)
   if constexpr (sizeof(LT) == 4 && LARGE) {
     tc_rect<4>((float*)M, ld, kb, nb, kb + nb, S, kb + nb, S);
-    __syncthreads();
+    csync();
     return;
   }
 #endif
-  if (!LARGE) {
+  if constexpr (!LARGE) {
     switch ((ncol + 31) >> 5) {
       case 1: trailing_update_ng<LT, 1, 4>(M, S, ld, kb, nb); break;
-      case 2: trailing_update_ng<LT, 2, 4>(M, S, ld, kb, nb); break;
-      case 3: trailing_update_ng<LT, 3, 4>(M, S, ld, kb, nb); break;
-      case 4: trailing_update_ng<LT, 4, 4>(M, S, ld, kb, nb); break;
-      case 5: trailing_update_ng<LT, 5, 4>(M, S, ld, kb, nb); break;
-      case 6: trailing_update_ng<LT, 6, 4>(M, S, ld, kb, nb); break;
-      case 7: trailing_update_ng<LT, 7, 4>(M, S, ld, kb, nb); break;
-      default: trailing_update_ng<LT, 8, 4>(M, S, ld, kb, nb); break;
+      case 2: if constexpr (kMaxColRegs >= 2) trailing_update_ng<LT, 2, 4>(M, S, ld, kb, nb); break;
+      case 3: if constexpr (kMaxColRegs >= 3) trailing_update_ng<LT, 3, 4>(M, S, ld, kb, nb); break;
+      case 4: if constexpr (kMaxColRegs >= 4) trailing_update_ng<LT, 4, 4>(M, S, ld, kb, nb); break;
+      case 5: if constexpr (kMaxColRegs >= 5) trailing_update_ng<LT, 5, 4>(M, S, ld, kb, nb); break;
+      case 6: if constexpr (kMaxColRegs >= 6) trailing_update_ng<LT, 6, 4>(M, S, ld, kb, nb); break;
+      case 7: if constexpr (kMaxColRegs >= 7) trailing_update_ng<LT, 7, 4>(M, S, ld, kb, nb); break;
+      default: if constexpr (kMaxColRegs >= 8) trailing_update_ng<LT, 8, 4>(M, S, ld, kb, nb); break;
     }
-    __syncthreads();
+    csync();
     return;
   }
   switch ((ncol + 31) >> 5) {
@@ -1014,7 +1288,7 @@ __device__ __forceinline__ void trailing_update(LT* M, int S, int ld, int kb, in
     case 15: trailing_update_ng<LT, 15, 2>(M, S, ld, kb, nb); break;
     default: trailing_update_ng<LT, 16, 2>(M, S, ld, kb, nb); break;
   }
-  __syncthreads();
+  csync();
 }
 
 // U_bb^{-1} of every diagonal block, in place (strict upper part; the
@@ -1049,7 +1323,7 @@ __device__ __forceinline__ void invert_upper_block(LT* U, const LT* invd, int ld
 // in place) and the still-original column j; lanes take the rows r < j.
 template <typename LT>
 __device__ void invert_upper_blocks_cols(LT* M, const LT* invd, int S, int ld) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid() >> 5, lane = tid() & 31;
   const int nblk = (S + NB - 1) / NB;
   for (int b = warp; b < nblk; b += NW) {
     const int kb = b * NB, nb = min(NB, S - kb);
@@ -1073,7 +1347,7 @@ __device__ void invert_upper_blocks_cols(LT* M, const LT* invd, int S, int ld) {
       __syncwarp();
     }
   }
-  __syncthreads();
+  csync();
 }
 
 template <typename LT>
@@ -1082,14 +1356,14 @@ __device__ void invert_upper_blocks(LT* M, const LT* invd, int S, int ld) {
     invert_upper_blocks_cols<LT>(M, invd, S, ld);
     return;
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid() >> 5, lane = tid() & 31;
   const int nblk = (S + NB - 1) / NB;
   for (int b = warp; b < nblk; b += NW) {
     const int kb = b * NB, nb = min(NB, S - kb);
     if (nb == NB) invert_upper_block<LT, true>(M + kb * ld + kb, invd + kb, ld, nb, lane);
     else invert_upper_block<LT, false>(M + kb * ld + kb, invd + kb, ld, nb, lane);
   }
-  __syncthreads();
+  csync();
 }
 
 // A22 -= L21 U12 for one of the leading panels [kb, kb+NB) of a network whose
@@ -1101,7 +1375,7 @@ __device__ void invert_upper_blocks(LT* M, const LT* invd, int S, int ld) {
 template <typename LT>
 __device__ void sparse_panel_update(LT* M, int S, int ld, int kb, const int* uptr, const int* ucol) {
   const int ke = kb + NB;
-  for (int i = ke + threadIdx.x; i < S; i += NT) {
+  for (int i = ke + tid(); i < S; i += NT) {
     LT* row = M + (size_t)i * ld;
     for (int c = 0; c < NB; ++c) {
       const LT l = row[kb + c];
@@ -1126,7 +1400,7 @@ __device__ void sparse_panel_update(LT* M, int S, int ld, int kb, const int* upt
       }
     }
   }
-  __syncthreads();
+  csync();
 }
 
 // FP32, matrix in global memory: panels in pairs, so that the trailing matrix
@@ -1155,11 +1429,11 @@ __device__ __noinline__ void lu_blocked_pairs(float* M, float* invd, int S, int 
     panel_u12<float, true>(M, S, ld, kb, NB);
     tc_rect<4>(M, ld, kb, NB, k2, S, k2, ke);   // P2's columns
     tc_rect<4>(M, ld, kb, NB, k2, ke, ke, S);   // P2's U rows (disjoint from the above)
-    __syncthreads();
+    csync();
     panel_factor_full_rows(M, invd, S, ld, k2);
     panel_u12<float, true>(M, S, ld, k2, NB);
     tc_rect<4>(M, ld, kb, 2 * NB, ke, S, ke, S);
-    __syncthreads();
+    csync();
   }
   for (; kb < S; kb += NB) {  // what is left: single panels
     const int nb = min(NB, S - kb);
@@ -1171,7 +1445,7 @@ __device__ __noinline__ void lu_blocked_pairs(float* M, float* invd, int S, int 
       panel_u12<float, false>(M, S, ld, kb, nb);
     }
     tc_rect<4>(M, ld, kb, nb, kb + nb, S, kb + nb, S);
-    __syncthreads();
+    csync();
   }
   invert_upper_blocks<float>(M, invd, S, ld);
 }
@@ -1211,7 +1485,7 @@ __device__ void lu_blocked(LT* M, LT* invd, int S, int ld, int nsp = 0, const in
 template <typename LT, bool FULL>
 __device__ __forceinline__ void rows_minus_block(const LT* M, int ld, const LT* vb, int nb, LT* v, int i0, int i1) {
   // v[i] -= sum_c M[i][c] vb[c] for rows i in [i0, i1); M points at column kb
-  for (int i = i0 + threadIdx.x; i < i1; i += NT) {
+  for (int i = i0 + tid(); i < i1; i += NT) {
     const LT* row = M + i * ld;
     LT p0 = v[i], p1 = LT(0), p2 = LT(0), p3 = LT(0);
 #pragma unroll
@@ -1227,7 +1501,7 @@ __device__ __forceinline__ void rows_minus_block(const LT* M, int ld, const LT* 
 
 template <typename LT>
 __device__ void solve_blocked(const LT* M, const LT* invd, int S, int ld, LT* v) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int warp = tid() >> 5, lane = tid() & 31;
   for (int kb = 0; kb < S; kb += NB) {
     const int nb = min(NB, S - kb), ke = kb + nb;
     if (warp == 0) {
@@ -1242,12 +1516,12 @@ __device__ void solve_blocked(const LT* M, const LT* invd, int S, int ld, LT* v)
       __syncwarp();
       if (lane < nb) v[kb + lane] = acc;
     }
-    __syncthreads();
+    csync();
     if (nb == NB)
       rows_minus_block<LT, true>(M + kb, ld, v + kb, nb, v, ke, S);
     else
       rows_minus_block<LT, false>(M + kb, ld, v + kb, nb, v, ke, S);
-    __syncthreads();
+    csync();
   }
   for (int kb = ((S - 1) / NB) * NB; kb >= 0; kb -= NB) {
     const int nb = min(NB, S - kb);
@@ -1263,12 +1537,12 @@ __device__ void solve_blocked(const LT* M, const LT* invd, int S, int ld, LT* v)
       __syncwarp();
       if (lane < nb) v[kb + lane] = acc;
     }
-    __syncthreads();
+    csync();
     if (nb == NB)
       rows_minus_block<LT, true>(M + kb, ld, v + kb, nb, v, 0, kb);
     else
       rows_minus_block<LT, false>(M + kb, ld, v + kb, nb, v, 0, kb);
-    __syncthreads();
+    csync();
   }
 }
 
@@ -1278,6 +1552,7 @@ struct Smem {
   void* M;
   void* invd;
   double *D, *y, *yp, *dv, *f, *wsc, *psi, *dy, *w, *tmp, *r, *part, *red, *Tm;
+  Scratch sc;    // reductions in red
   float* v32;
   int* pstage;   // staged pivot lists (FP64 shared-memory solver), or none
   PivLists piv;  // the lists the LU reads
@@ -1285,8 +1560,12 @@ struct Smem {
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
+// Lean: the rates r and the segment sums part live in the CTA's workspace (they
+// are dead outside a right-hand side, so they take the place of the Jacobian's
+// reaction partials: nseg <= R), and f shares its storage with w, psi with tmp.
+// Two CTAs then fit an SM up to 111 species in FP64 and 152 mixed.
 __host__ __device__ inline size_t layout(int S, int R, int nseg, bool mixed, bool gm, unsigned char* base, Smem* s,
-                                         int piv_ints = 0) {
+                                         int piv_ints = 0, bool lean = false) {
   const size_t lt = mixed ? sizeof(float) : sizeof(double);
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -1305,14 +1584,15 @@ __host__ __device__ inline size_t layout(int S, int R, int nseg, bool mixed, boo
   t.wsc = (double*)take(S * 8);
   t.psi = (double*)take(S * 8);
   t.dy = (double*)take(S * 8);
-  t.w = (double*)take(S * 8);
-  t.tmp = (double*)take(S * 8);
-  t.r = (double*)take((size_t)R * 8);
-  t.part = (double*)take((size_t)nseg * 8);
+  t.w = lean ? t.f : (double*)take(S * 8);
+  t.tmp = lean ? t.psi : (double*)take(S * 8);
+  t.r = lean ? nullptr : (double*)take((size_t)R * 8);
+  t.part = lean ? nullptr : (double*)take((size_t)nseg * 8);
   t.red = (double*)take(128 * 8);  // block sums; the solves' look-ahead partials
   t.Tm = (double*)take(kMaxOrder * kMaxOrder * 8);
   t.v32 = (float*)take(mixed ? S * 4 : 0);
   t.pstage = (int*)take((size_t)piv_ints * 4);
+  t.sc = Scratch{t.red, 0};
   if (s) *s = t;
   return off;
 }
@@ -1328,13 +1608,13 @@ __device__ void stage_pivots(const DevNet& n, Smem& s) {
   int* up = lp + (kd + 1);
   int* l = up + (kd + 1);
   int* u = l + nl;
-  for (int i = threadIdx.x; i <= kd; i += NT) {
+  for (int i = tid(); i <= kd; i += NT) {
     lp[i] = n.piv_lptr[i];
     up[i] = n.piv_uptr[i];
   }
-  for (int i = threadIdx.x; i < nl; i += NT) l[i] = n.piv_l[i];
-  for (int i = threadIdx.x; i < nu; i += NT) u[i] = n.piv_u[i];
-  __syncthreads();
+  for (int i = tid(); i < nl; i += NT) l[i] = n.piv_l[i];
+  for (int i = tid(); i < nu; i += NT) u[i] = n.piv_u[i];
+  csync();
   s.piv = PivLists{n.S, kd, lp, l, up, u};
 }
 
@@ -1350,30 +1630,38 @@ static __constant__ double c_binom[kMaxOrder + 1][kMaxOrder + 1] = {{1, 0, 0, 0,
                                                              {1, 2, 1, 0, 0, 0}, {1, 3, 3, 1, 0, 0},
                                                              {1, 4, 6, 4, 1, 0}, {1, 5, 10, 10, 5, 1}};
 
-__device__ __forceinline__ double rescale_entry(int k, int j, double rho) {
-  double acc = 0.0;
-  for (int i = 0; i <= k; ++i) {
-    const double s = -i * rho;
+// T (q x q, rows k, stride kMaxOrder) by one warp: lanes first form the
+// products P(i, j) = prod_{m<j} (-i rho + m) of all i and j side by side (every
+// entry of column j needs those of i <= k; formed entry by entry they were a
+// serial chain of up to 70 FP64 instructions of 64 cycles), then lane (k, j)
+// sums its terms in order. P: 30 doubles of shared scratch.
+__device__ void rescale_matrix(int q, double rho, double* Tm, double* P) {
+  const int lane = tid() & 31;
+  if (lane < (kMaxOrder + 1) * kMaxOrder) {
+    const int i = lane / kMaxOrder, j = lane % kMaxOrder + 1;
+    // rounded operations: a contraction of -i rho + m would depend on unrolling
+    const double s = __dmul_rn((double)-i, rho);
     double p = 1.0;
-    for (int m = 0; m < j; ++m) p *= s + m;
-    acc = fma((i & 1) ? -c_binom[k][i] : c_binom[k][i], p, acc);
+    for (int m = 0; m < j; ++m) p = __dmul_rn(p, __dadd_rn(s, (double)m));
+    P[lane] = p;
   }
-  return acc * c_inv_fact[j];
+  __syncwarp();
+  if (lane < q * q) {
+    const int k = lane / q + 1, j = lane % q + 1;
+    double acc = 0.0;
+    for (int i = 0; i <= k; ++i)
+      acc = fma((i & 1) ? -c_binom[k][i] : c_binom[k][i], P[i * kMaxOrder + j - 1], acc);
+    Tm[(k - 1) * kMaxOrder + (j - 1)] = acc * c_inv_fact[j];
+  }
 }
 
 // D[1..q] <- T(rho) D[1..q], T[k][j] = sum_i (-1)^i C(k,i) C(-i rho + j - 1, j):
-// the differences of the interpolating polynomial on the new spacing. The
-// q x q matrix is computed by one warp (lane = (k, j)).
-__device__ void rescale(double* D, int S, int q, double rho, double* Tm) {
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    if (lane < q * q) {
-      const int k = lane / q + 1, j = lane % q + 1;
-      Tm[(k - 1) * kMaxOrder + (j - 1)] = rescale_entry(k, j, rho);
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < S; i += NT) {
+// the differences of the interpolating polynomial on the new spacing.
+__device__ void rescale(double* D, int S, int q, double rho, double* Tm, Scratch& sc) {
+  double* P = sc.next();
+  if (tid() < 32) rescale_matrix(q, rho, Tm, P);
+  csync();
+  for (int i = tid(); i < S; i += NT) {
     double old[kMaxOrder];
 #pragma unroll
     for (int j = 0; j < kMaxOrder; ++j) old[j] = j < q ? D[(j + 1) * S + i] : 0.0;
@@ -1385,7 +1673,39 @@ __device__ void rescale(double* D, int S, int q, double rho, double* Tm) {
       D[(k + 1) * S + i] = acc;
     }
   }
-  __syncthreads();
+  csync();
+}
+
+// Order and step change after q+1 equal steps: the error estimates at q-1, q
+// and q+1 (err is that of order q), the growth factors err_k^(-1/(k+1)) in
+// three lanes of one warp, and the order of the largest. Returns the step
+// factor. Two barriers.
+__device__ double next_order(const double* D, const double* wsc, double err, int S, int* q_io, Scratch& sc) {
+  const int q = *q_io;
+  double* slot = sc.next();
+  const bool down = q > 1, up = q < kMaxOrder;
+  const double ad = 1.0 / q, au = 1.0 / (q + 2);
+  if (down) chunk_sums([&](int i) { return ad * D[q * S + i] * wsc[i]; }, S, slot);
+  if (up) chunk_sums([&](int i) { return au * D[(q + 2) * S + i] * wsc[i]; }, S, slot + 16);
+  csync();
+  if (tid() < 32) {
+    const int lane = tid();
+    double e = INFINITY;
+    if (lane == 0 && down) e = sqrt(chunk_total(slot, S) / S);
+    if (lane == 1) e = err;
+    if (lane == 2 && up) e = sqrt(chunk_total(slot + 16, S) / S);
+    // every lane past 2 repeats lane 1's work
+    const int p = lane < 3 ? q + lane : q + 1;
+    if (lane > 2) e = err;
+    const double g = e == 0.0 ? INFINITY : pow(e, -1.0 / p);
+    if (lane < 3) slot[32 + lane] = g;
+  }
+  csync();
+  int best = 0;
+  if (slot[33] > slot[32 + best]) best = 1;
+  if (slot[34] > slot[32 + best]) best = 2;
+  *q_io = q + best - 1;
+  return fmin(10.0, 0.9 * slot[32 + best]);
 }
 
 template <typename LT, bool GM>
@@ -1401,12 +1721,10 @@ struct Cell {
   cbx_cell_stats* st;  // shared-memory counters, updated by thread 0 only
 };
 
-// Solve (I - cJ) dy = w with the factored matrix in shared memory.
+// Solve (I - cJ) dy = w with the factored matrix; w is in dy on entry.
 template <bool GM>
 __device__ void linear_solve(Cell<double, GM>& c, double cc, const double* w, double* dy) {
   const int S = c.n.S;
-  for (int i = threadIdx.x; i < S; i += NT) dy[i] = w[i];
-  __syncthreads();
   if constexpr (GM) {
     solve_blocked<double>(c.M, (const double*)c.s.invd, S, lead_dim(S), dy);
   } else {
@@ -1417,7 +1735,7 @@ __device__ void linear_solve(Cell<double, GM>& c, double cc, const double* w, do
 
 // FP32 LU solve, then FP64 residual w - (dy - c J dy) against the FP64
 // Jacobian and FP32 correction solves until the weighted RMS of the
-// correction is <= refine_tol or max_refine sweeps.
+// correction is <= refine_tol or max_refine sweeps. v32 holds w on entry.
 template <bool GM>
 __device__ void linear_solve(Cell<float, GM>& c, double cc, const double* w, double* dy) {
   const int S = c.n.S;
@@ -1425,31 +1743,37 @@ __device__ void linear_solve(Cell<float, GM>& c, double cc, const double* w, dou
   const float* invd = (const float*)c.s.invd;
   float* v = c.s.v32;
   const int ld = lead_dim(S);
-  for (int i = threadIdx.x; i < S; i += NT) v[i] = (float)w[i];
-  __syncthreads();
   solve_blocked<float>(M, invd, S, ld, v);
-  for (int i = threadIdx.x; i < S; i += NT) dy[i] = (double)v[i];
-  __syncthreads();
+  for (int i = tid(); i < S; i += NT) dy[i] = (double)v[i];
+  csync();
   for (int sweep = 0; sweep < c.a.max_refine; ++sweep) {
-    for (int i = threadIdx.x; i < S; i += NT) {
+    for (int i = tid(); i < S; i += NT) {
       double acc = 0.0;
       const int e1 = c.n.jrow_ptr[i + 1];
       for (int e = c.n.jrow_ptr[i]; e < e1; ++e) acc = fma(c.Jv[e], dy[c.n.jcol[e]], acc);
       const double res = w[i] - (dy[i] - cc * acc);
       v[i] = (float)res;
     }
-    __syncthreads();
+    csync();
     solve_blocked<float>(M, invd, S, ld, v);
-    double sq = 0.0;
-    for (int i = threadIdx.x; i < S; i += NT) {
-      const double corr = (double)v[i];
-      dy[i] += corr;
-      const double t = corr * c.s.wsc[i];
-      sq = fma(t, t, sq);
+    double* slot = c.s.sc.next();
+    chunk_sums(
+        [&](int i) {
+          const double corr = (double)v[i];
+          dy[i] += corr;
+          return corr * c.s.wsc[i];
+        },
+        S, slot);
+    csync();
+    if (tid() < 32) {
+      const bool more = sqrt(chunk_total(slot, S) / S) > c.a.refine_tol;
+      if (tid() == 0) {
+        c.st->refine_sweeps++;
+        slot[kChunks] = more;
+      }
     }
-    if (threadIdx.x == 0) c.st->refine_sweeps++;
-    const double nrm = sqrt(block_sum(sq, c.s.red) / S);
-    if (!(nrm > c.a.refine_tol)) break;
+    csync();
+    if (slot[kChunks] == 0.0) break;
   }
 }
 
@@ -1464,7 +1788,7 @@ __device__ void factor(Cell<LT, GM>& c, double cc) {
     else
       lu_crout64(c.s.piv, c.M, (double*)c.s.invd);
   }
-  if (threadIdx.x == 0) c.st->lu_factors++;
+  if (tid() == 0) c.st->lu_factors++;
 }
 
 // Simplified Newton on d - c f(yp + d) + psi = 0. Leaves y = yp + d, dv = d.
@@ -1472,40 +1796,62 @@ template <typename LT, bool GM>
 __device__ bool newton(Cell<LT, GM>& c, double cc, int* iters) {
   const int S = c.n.S;
   Smem& s = c.s;
-  for (int i = threadIdx.x; i < S; i += NT) {
+  for (int i = tid(); i < S; i += NT) {
     s.y[i] = s.yp[i];
     s.dv[i] = 0.0;
   }
-  __syncthreads();
-  double dy_old = 0.0, rate = 0.0;
+  csync();
+  double dy_old = 0.0;  // warp 0's
   bool conv = false;
   for (int k = 0; k < kNewtonMaxIter; ++k) {
     *iters = k + 1;
     rhs(c.n, c.kap, s.y, s.f, s.r, s.part);
-    if (threadIdx.x == 0) c.st->rhs_evals++;
+    if (tid() == 0) c.st->rhs_evals++;
     int bad = 0;
-    for (int i = threadIdx.x; i < S; i += NT) bad |= !isfinite(s.f[i]);
-    if (__syncthreads_or(bad)) break;
-    for (int i = threadIdx.x; i < S; i += NT) s.w[i] = cc * s.f[i] - s.psi[i] - s.dv[i];
-    __syncthreads();
-    linear_solve(c, cc, s.w, s.dy);
-    const double dyn = wrms(s.dy, s.wsc, 1.0, S, s.red);
-    if (k > 0) {
-      rate = dyn / dy_old;
-      double rp = 1.0;
-      for (int m = 0; m < kNewtonMaxIter - k; ++m) rp *= rate;
-      if (rate >= 1.0 || rp / (1.0 - rate) * dyn > c.a.newton_tol) break;
+    for (int i = tid(); i < S; i += NT) {
+      const double f = s.f[i], w = cc * f - s.psi[i] - s.dv[i];
+      bad |= !isfinite(f);
+      if constexpr (sizeof(LT) == 8) {
+        s.dy[i] = w;  // solved in place
+      } else {
+        s.w[i] = w;
+        s.v32[i] = (float)w;
+      }
     }
-    for (int i = threadIdx.x; i < S; i += NT) {
+    if (csync_or(bad)) break;
+    linear_solve(c, cc, s.w, s.dy);
+    // warp 0: |dy|, the rate test and the convergence test
+    double* slot = s.sc.next();
+    chunk_sums([&](int i) { return s.dy[i] * s.wsc[i]; }, S, slot);
+    csync();
+    if (tid() < 32) {
+      const double dyn = sqrt(chunk_total(slot, S) / S);
+      double verdict = 0.0;  // 1: no contraction; 2: converged
+      if (k > 0) {
+        const double rate = dyn / dy_old;
+        double rp = 1.0;
+        for (int m = 0; m < kNewtonMaxIter - k; ++m) rp *= rate;
+        // both quotients by one division: even lanes rate / (1 - rate), odd ones rp / (1 - rate)
+        const double test = ((tid() & 1) ? rp : rate) / (1.0 - rate) * dyn;
+        if (rate >= 1.0 || __shfl_sync(FULL, test, 1) > c.a.newton_tol) verdict = 1.0;
+        else if (__shfl_sync(FULL, test, 0) < c.a.newton_tol) verdict = 2.0;
+      }
+      if (dyn == 0.0 && verdict == 0.0) verdict = 2.0;
+      if (tid() == 0) slot[kChunks] = verdict;
+      dy_old = dyn;
+    }
+    csync();
+    const double verdict = slot[kChunks];
+    if (verdict == 1.0) break;
+    for (int i = tid(); i < S; i += NT) {
       s.y[i] += s.dy[i];
       s.dv[i] += s.dy[i];
     }
-    __syncthreads();
-    if (dyn == 0.0 || (k > 0 && rate / (1.0 - rate) * dyn < c.a.newton_tol)) {
+    csync();
+    if (verdict == 2.0) {
       conv = true;
       break;
     }
-    dy_old = dyn;
   }
   return conv;
 }
@@ -1522,7 +1868,7 @@ __device__ void rec_op(const SolveArgs& a, int cell, Recorder& r, int kind, int 
     r.full = true;
     return;
   }
-  if (threadIdx.x == 0) {
+  if (tid() == 0) {
     const size_t o = (size_t)cell * a.tape.cap_ops + r.nops;
     a.tape.ops_kq[o] = (kind << 8) | q;
     a.tape.ops_v[o] = v;
@@ -1538,8 +1884,8 @@ __device__ void rec_step(const SolveArgs& a, int cell, Recorder& r, int q, doubl
     return;
   }
   double* dst = a.tape.ys + ((size_t)cell * a.tape.cap_steps + r.nsteps) * S;
-  for (int i = threadIdx.x; i < S; i += NT) dst[i] = y[i];
-  if (threadIdx.x == 0) a.tape.ts[(size_t)cell * a.tape.cap_steps + r.nsteps] = t_new;
+  for (int i = tid(); i < S; i += NT) dst[i] = y[i];
+  if (tid() == 0) a.tape.ts[(size_t)cell * a.tape.cap_steps + r.nsteps] = t_new;
   rec_op(a, cell, r, kOpStep, q, h);
   r.nsteps++;
 }
@@ -1587,7 +1933,7 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
   LT* M = GM ? (LT*)(ws + (3LL * n.R + n.nnzJ + 31) / 32 * 32) : (LT*)s.M;
   __shared__ cbx_cell_stats s_stats;
   Cell<LT, GM> c{a, n, s, M, ws, ws + n.R, ws + 3 * n.R, &s_stats};
-  if (threadIdx.x == 0) {
+  if (tid() == 0) {
     *c.st = cbx_cell_stats{};
     c.st->t_begin_ns = (long long)globaltimer();
   }
@@ -1596,22 +1942,22 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
   int status = CBX_CELL_OK;
   Recorder rec;
   rec.on = a.tape.nops != nullptr;
-  for (int i = threadIdx.x; i < S; i += NT) s.y[i] = a.x0[(size_t)__ldg(n.perm + i) * a.C + cell];
+  for (int i = tid(); i < S; i += NT) s.y[i] = a.x0[(size_t)__ldg(n.perm + i) * a.C + cell];
   if (!(p.n_H > 0.0) || !(p.T > 0.0) || !isfinite(p.n_H) || !isfinite(p.T) || !isfinite(p.A_V) ||
       !isfinite(p.G0) || !isfinite(p.zeta) || (a.track && !track_valid(a.track, a.K, cell)) ||
       !(cell_t_end(a, cell) >= a.t0) || !isfinite(cell_t_end(a, cell))) {
     status = CBX_CELL_BAD_INPUT;
-    __syncthreads();
-    for (int i = threadIdx.x; i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = s.y[i];
+    csync();
+    for (int i = tid(); i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = s.y[i];
   } else {
     rate_coefficients(n, a.alpha, p, c.kap);
-    __syncthreads();
+    csync();
     // with a track, the coefficients follow phi(t) to every time f or J is evaluated at
     double t_rates = a.t0;
     auto rates_at = [&](double tt) {
       if (a.track && tt != t_rates) {
         rate_coefficients(n, a.alpha, track_params(a.track, a.K, cell, tt), c.kap);
-        __syncthreads();
+        csync();
         t_rates = tt;
       }
     };
@@ -1619,25 +1965,25 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
     double* D = s.D;
     // f0 and the initial step (Hairer, Norsett & Wanner I, II.4, p = 1)
     rhs(n, c.kap, s.y, s.f, s.r, s.part);
-    if (threadIdx.x == 0) c.st->rhs_evals++;
-    for (int i = threadIdx.x; i < S; i += NT) s.wsc[i] = 1.0 / (atol + rtol * fabs(s.y[i]));
-    __syncthreads();
-    const double d0 = wrms(s.y, s.wsc, 1.0, S, s.red);
-    const double d1 = wrms(s.f, s.wsc, 1.0, S, s.red);
+    if (tid() == 0) c.st->rhs_evals++;
+    for (int i = tid(); i < S; i += NT) s.wsc[i] = __drcp_rn(atol + rtol * fabs(s.y[i]));
+    csync();
+    const double d0 = wrms(s.y, s.wsc, 1.0, S, s.sc);
+    const double d1 = wrms(s.f, s.wsc, 1.0, S, s.sc);
     const double h0 = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
-    for (int i = threadIdx.x; i < S; i += NT) s.tmp[i] = s.y[i] + h0 * s.f[i];
-    __syncthreads();
+    for (int i = tid(); i < S; i += NT) s.tmp[i] = s.y[i] + h0 * s.f[i];
+    csync();
     rates_at(a.t0 + h0);
     rhs(n, c.kap, s.tmp, s.dy, s.r, s.part);
-    if (threadIdx.x == 0) c.st->rhs_evals++;
-    for (int i = threadIdx.x; i < S; i += NT) s.tmp[i] = s.dy[i] - s.f[i];
-    __syncthreads();
-    const double d2 = wrms(s.tmp, s.wsc, 1.0, S, s.red) / h0;
+    if (tid() == 0) c.st->rhs_evals++;
+    for (int i = tid(); i < S; i += NT) s.tmp[i] = s.dy[i] - s.f[i];
+    csync();
+    const double d2 = wrms(s.tmp, s.wsc, 1.0, S, s.sc) / h0;
     const double dm = fmax(d1, d2);
     const double h1 = dm <= 1e-15 ? fmax(1e-6, h0 * 1e-3) : sqrt(0.01 / dm);
     double t = a.t0;
     double h = fmin(fmin(100.0 * h0, h1), t_end - t);
-    for (int i = threadIdx.x; i < S; i += NT) {
+    for (int i = tid(); i < S; i += NT) {
       D[i] = s.y[i];
       D[S + i] = h * s.f[i];
       for (int r = 2; r < kDiffRows; ++r) D[r * S + i] = 0.0;
@@ -1645,10 +1991,9 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
     rec_op(a, cell, rec, kOpInit, 1, h);
     rates_at(a.t0);
     jacobian(n, c.kap, s.y, c.g, c.Jv);
-    if (threadIdx.x == 0) c.st->jac_evals++;
+    if (tid() == 0) c.st->jac_evals++;
     int q = 1, n_equal = 0;
     bool jac_current = true, lu_valid = false;
-    double* slot = s.red + 40;
     while (t < t_end) {
       bool accepted = false;
       double t_new = t, err = 0.0;
@@ -1665,23 +2010,23 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
         t_new = t + h;
         if (t_new > t_end) {
           t_new = t_end;
-          rescale(D, S, q, (t_end - t) / h, s.Tm);
+          rescale(D, S, q, (t_end - t) / h, s.Tm, s.sc);
           rec_op(a, cell, rec, kOpRescale, q, (t_end - t) / h);
           n_equal = 0;
           lu_valid = false;
           h = t_end - t;
         }
         const double gq = a.gam[q];
-        for (int i = threadIdx.x; i < S; i += NT) {
+        for (int i = tid(); i < S; i += NT) {
           double yp = 0.0;
           for (int j = 0; j <= q; ++j) yp += D[j * S + i];
           double ps = 0.0;
           for (int j = 1; j <= q; ++j) ps = fma(a.gam[j], D[j * S + i], ps);
           s.yp[i] = yp;
           s.psi[i] = ps / gq;
-          s.wsc[i] = 1.0 / (atol + rtol * fabs(yp));
+          s.wsc[i] = __drcp_rn(atol + rtol * fabs(yp));
         }
-        __syncthreads();
+        csync();
         const double cc = h / gq;
         bool conv = false;
         int iters = 0;
@@ -1692,29 +2037,29 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
             lu_valid = true;
           }
           conv = newton(c, cc, &iters);
-          if (threadIdx.x == 0) c.st->newton_iters += iters;
+          if (tid() == 0) c.st->newton_iters += iters;
           if (conv || jac_current) break;
           jacobian(n, c.kap, s.yp, c.g, c.Jv);
-          if (threadIdx.x == 0) c.st->jac_evals++;
+          if (tid() == 0) c.st->jac_evals++;
           jac_current = true;
           lu_valid = false;
         }
         if (!conv) {
-          if (threadIdx.x == 0) c.st->newton_fails++;
-          rescale(D, S, q, 0.5, s.Tm);
+          if (tid() == 0) c.st->newton_fails++;
+          rescale(D, S, q, 0.5, s.Tm, s.sc);
           rec_op(a, cell, rec, kOpRescale, q, 0.5);
           h *= 0.5;
           n_equal = 0;
           lu_valid = false;
           continue;
         }
-        for (int i = threadIdx.x; i < S; i += NT) s.wsc[i] = 1.0 / (atol + rtol * fabs(s.y[i]));
-        __syncthreads();
-        err = wrms(s.dv, s.wsc, 1.0 / (q + 1), S, s.red);
+        for (int i = tid(); i < S; i += NT) s.wsc[i] = __drcp_rn(atol + rtol * fabs(s.y[i]));
+        csync();
+        err = wrms(s.dv, s.wsc, 1.0 / (q + 1), S, s.sc);
         if (err > 1.0) {
-          if (threadIdx.x == 0) c.st->error_fails++;
-          const double fac = fmax(0.2, 0.9 * uniform_pow(err, -1.0 / (q + 1), slot));
-          rescale(D, S, q, fac, s.Tm);
+          if (tid() == 0) c.st->error_fails++;
+          const double fac = fmax(0.2, 0.9 * uniform_pow(err, -1.0 / (q + 1), s.sc));
+          rescale(D, S, q, fac, s.Tm, s.sc);
           rec_op(a, cell, rec, kOpRescale, q, fac);
           h *= fac;
           n_equal = 0;
@@ -1725,46 +2070,36 @@ __device__ void solve_cell(const SolveArgs& a, int cell, Smem& s, double* ws) {
       }
       if (!accepted) break;
       rec_step(a, cell, rec, q, h, t_new, s.y, S);
-      if (threadIdx.x == 0) c.st->steps++;
+      if (tid() == 0) c.st->steps++;
       t = t_new;
       jac_current = false;
       n_equal++;
-      for (int i = threadIdx.x; i < S; i += NT) {
+      for (int i = tid(); i < S; i += NT) {
         const double d = s.dv[i];
         D[(q + 2) * S + i] = d - D[(q + 1) * S + i];
         D[(q + 1) * S + i] = d;
         for (int j = q; j >= 0; --j) D[j * S + i] += D[(j + 1) * S + i];
       }
-      __syncthreads();
+      csync();
       if (n_equal < q + 1) continue;
-      const double em = q > 1 ? wrms(D + q * S, s.wsc, 1.0 / q, S, s.red) : INFINITY;
-      const double ep = q < kMaxOrder ? wrms(D + (q + 2) * S, s.wsc, 1.0 / (q + 2), S, s.red) : INFINITY;
-      double fc[3];
-      fc[0] = growth(em, q, slot);
-      fc[1] = growth(err, q + 1, slot);
-      fc[2] = growth(ep, q + 2, slot);
-      int best = 0;
-      if (fc[1] > fc[best]) best = 1;
-      if (fc[2] > fc[best]) best = 2;
-      q += best - 1;
-      const double fac = fmin(10.0, 0.9 * fc[best]);
-      rescale(D, S, q, fac, s.Tm);
+      const double fac = next_order(D, s.wsc, err, S, &q, s.sc);
+      rescale(D, S, q, fac, s.Tm, s.sc);
       rec_op(a, cell, rec, kOpRescale, q, fac);
       h *= fac;
       n_equal = 0;
       lu_valid = false;
     }
-    for (int i = threadIdx.x; i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = D[i];
+    for (int i = tid(); i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = D[i];
   }
   if (rec.on && rec.full && status == CBX_CELL_OK) status = CBX_CELL_TAPE_FULL;
-  if (threadIdx.x == 0) {
+  if (tid() == 0) {
     if (rec.on) a.tape.nops[cell] = rec.nops;
     a.status[cell] = status;
     c.st->attempts = attempts;
     c.st->t_end_ns = (long long)globaltimer();
     if (a.stats) a.stats[cell] = *c.st;
   }
-  __syncthreads();
+  csync();
 }
 // ---------------------------------------------------------------- ESDIRK
 //
@@ -1790,7 +2125,7 @@ __device__ void solve_cell_rk(const SolveArgs& a, int cell, Smem& s, double* ws)
   LT* M = GM ? (LT*)(ws + (3LL * n.R + n.nnzJ + 31) / 32 * 32) : (LT*)s.M;
   __shared__ cbx_cell_stats s_stats;
   Cell<LT, GM> c{a, n, s, M, ws, ws + n.R, ws + 3 * n.R, &s_stats};
-  if (threadIdx.x == 0) {
+  if (tid() == 0) {
     *c.st = cbx_cell_stats{};
     c.st->t_begin_ns = (long long)globaltimer();
   }
@@ -1800,50 +2135,49 @@ __device__ void solve_cell_rk(const SolveArgs& a, int cell, Smem& s, double* ws)
   double* F = s.D;           // f_1..f_5, rows 0..4
   double* yn = s.D + 5 * S;  // y_n
   double* yprev = s.D + 6 * S;
-  for (int i = threadIdx.x; i < S; i += NT) yn[i] = a.x0[(size_t)__ldg(n.perm + i) * a.C + cell];
+  for (int i = tid(); i < S; i += NT) yn[i] = a.x0[(size_t)__ldg(n.perm + i) * a.C + cell];
   if (!(p.n_H > 0.0) || !(p.T > 0.0) || !isfinite(p.n_H) || !isfinite(p.T) || !isfinite(p.A_V) ||
       !isfinite(p.G0) || !isfinite(p.zeta) || (a.track && !track_valid(a.track, a.K, cell)) ||
       !(cell_t_end(a, cell) >= a.t0) || !isfinite(cell_t_end(a, cell))) {
     status = CBX_CELL_BAD_INPUT;
-    __syncthreads();
-    for (int i = threadIdx.x; i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = yn[i];
+    csync();
+    for (int i = tid(); i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = yn[i];
   } else {
     rate_coefficients(n, a.alpha, p, c.kap);
-    __syncthreads();
+    csync();
     double t_rates = a.t0;
     auto rates_at = [&](double tt) {
       if (a.track && tt != t_rates) {
         rate_coefficients(n, a.alpha, track_params(a.track, a.K, cell, tt), c.kap);
-        __syncthreads();
+        csync();
         t_rates = tt;
       }
     };
     const double rtol = a.rtol, atol = a.atol, t_end = cell_t_end(a, cell);
     const double gamma = a.rk_a[1][1];
-    double* slot = s.red + 40;
     // f_1 and the initial step (Hairer, Norsett & Wanner I, II.4, p = 3)
     rhs(n, c.kap, yn, F, s.r, s.part);
-    if (threadIdx.x == 0) c.st->rhs_evals++;
-    for (int i = threadIdx.x; i < S; i += NT) s.wsc[i] = 1.0 / (atol + rtol * fabs(yn[i]));
-    __syncthreads();
-    const double d0 = wrms(yn, s.wsc, 1.0, S, s.red);
-    const double d1 = wrms(F, s.wsc, 1.0, S, s.red);
+    if (tid() == 0) c.st->rhs_evals++;
+    for (int i = tid(); i < S; i += NT) s.wsc[i] = __drcp_rn(atol + rtol * fabs(yn[i]));
+    csync();
+    const double d0 = wrms(yn, s.wsc, 1.0, S, s.sc);
+    const double d1 = wrms(F, s.wsc, 1.0, S, s.sc);
     const double h0 = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
-    for (int i = threadIdx.x; i < S; i += NT) s.tmp[i] = yn[i] + h0 * F[i];
-    __syncthreads();
+    for (int i = tid(); i < S; i += NT) s.tmp[i] = yn[i] + h0 * F[i];
+    csync();
     rates_at(a.t0 + h0);
     rhs(n, c.kap, s.tmp, s.dy, s.r, s.part);
-    if (threadIdx.x == 0) c.st->rhs_evals++;
-    for (int i = threadIdx.x; i < S; i += NT) s.tmp[i] = s.dy[i] - F[i];
-    __syncthreads();
-    const double d2 = wrms(s.tmp, s.wsc, 1.0, S, s.red) / h0;
+    if (tid() == 0) c.st->rhs_evals++;
+    for (int i = tid(); i < S; i += NT) s.tmp[i] = s.dy[i] - F[i];
+    csync();
+    const double d2 = wrms(s.tmp, s.wsc, 1.0, S, s.sc) / h0;
     const double dm = fmax(d1, d2);
-    const double h1 = dm <= 1e-15 ? fmax(1e-6, h0 * 1e-3) : uniform_pow(0.01 / dm, 0.25, slot);
+    const double h1 = dm <= 1e-15 ? fmax(1e-6, h0 * 1e-3) : uniform_pow(0.01 / dm, 0.25, s.sc);
     double t = a.t0;
     double h = fmin(fmin(100.0 * h0, h1), t_end - t);
     rates_at(a.t0);
     jacobian(n, c.kap, yn, c.g, c.Jv);
-    if (threadIdx.x == 0) c.st->jac_evals++;
+    if (tid() == 0) c.st->jac_evals++;
     bool jac_current = true, lu_valid = false;
     double lu_h = 0.0, err = 0.0;
     while (t < t_end) {
@@ -1868,102 +2202,106 @@ __device__ void solve_cell_rk(const SolveArgs& a, int cell, Smem& s, double* ws)
             lu_h = h;
           }
           failed = false;
-          for (int i = threadIdx.x; i < S; i += NT) {
+          for (int i = tid(); i < S; i += NT) {
             yprev[i] = yn[i];
-            s.wsc[i] = 1.0 / (atol + rtol * fabs(yn[i]));
+            s.wsc[i] = __drcp_rn(atol + rtol * fabs(yn[i]));
           }
-          __syncthreads();
+          csync();
           for (int st = 1; st < 5; ++st) {
             const double ti = t + a.rk_c[st] * h;
             // guess Y_{i-1}; psi = guess - known, known = y_n + h sum_{j<i} a_ij f_j
-            for (int i = threadIdx.x; i < S; i += NT) {
+            for (int i = tid(); i < S; i += NT) {
               double known = 0.0;
               for (int j = 0; j < st; ++j) known = fma(a.rk_a[st][j], F[j * S + i], known);
               known = fma(h, known, yn[i]);
               s.yp[i] = yprev[i];
               s.psi[i] = yprev[i] - known;
             }
-            __syncthreads();
+            csync();
             rates_at(ti);
             int iters = 0;
             const bool conv = newton(c, hg, &iters);
-            if (threadIdx.x == 0) c.st->newton_iters += iters;
+            if (tid() == 0) c.st->newton_iters += iters;
             if (!conv) {
               failed = true;
               break;
             }
             rhs(n, c.kap, s.y, F + st * S, s.r, s.part);
-            if (threadIdx.x == 0) c.st->rhs_evals++;
+            if (tid() == 0) c.st->rhs_evals++;
             if (st < 4) {  // after the last stage yprev keeps the embedded solution Y_4
-              for (int i = threadIdx.x; i < S; i += NT) yprev[i] = s.y[i];
-              __syncthreads();
+              for (int i = tid(); i < S; i += NT) yprev[i] = s.y[i];
+              csync();
             }
           }
           if (!failed || jac_current) break;
           rates_at(t);
           jacobian(n, c.kap, yn, c.g, c.Jv);
-          if (threadIdx.x == 0) c.st->jac_evals++;
+          if (tid() == 0) c.st->jac_evals++;
           jac_current = true;
           lu_valid = false;
         }
         if (failed) {
-          if (threadIdx.x == 0) c.st->newton_fails++;
+          if (tid() == 0) c.st->newton_fails++;
           h *= 0.5;
           continue;
         }
         // error estimate Y_5 - Y_4 (s.y = Y_5, yprev = Y_4), weights from |Y_5|
-        for (int i = threadIdx.x; i < S; i += NT) {
-          s.wsc[i] = 1.0 / (atol + rtol * fabs(s.y[i]));
+        for (int i = tid(); i < S; i += NT) {
+          s.wsc[i] = __drcp_rn(atol + rtol * fabs(s.y[i]));
           s.tmp[i] = s.y[i] - yprev[i];
         }
-        __syncthreads();
-        err = wrms(s.tmp, s.wsc, 1.0, S, s.red);
+        csync();
+        err = wrms(s.tmp, s.wsc, 1.0, S, s.sc);
         if (err > 1.0) {
-          if (threadIdx.x == 0) c.st->error_fails++;
-          h *= fmax(0.2, 0.9 * uniform_pow(err, -0.25, slot));
+          if (tid() == 0) c.st->error_fails++;
+          h *= fmax(0.2, 0.9 * uniform_pow(err, -0.25, s.sc));
           continue;
         }
         accepted = true;
       }
       if (!accepted) break;
-      if (threadIdx.x == 0) c.st->steps++;
+      if (tid() == 0) c.st->steps++;
       t = t + h;
-      for (int i = threadIdx.x; i < S; i += NT) {
+      for (int i = tid(); i < S; i += NT) {
         yn[i] = s.y[i];
         F[i] = F[4 * S + i];
       }
-      __syncthreads();
+      csync();
       jac_current = false;
-      const double fac = err == 0.0 ? 10.0 : 0.9 * uniform_pow(err, -0.25, slot);
+      const double fac = err == 0.0 ? 10.0 : 0.9 * uniform_pow(err, -0.25, s.sc);
       h *= fmin(10.0, fmax(0.2, fac));
     }
-    for (int i = threadIdx.x; i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = yn[i];
+    for (int i = tid(); i < S; i += NT) a.x_out[(size_t)__ldg(n.perm + i) * a.C + cell] = yn[i];
   }
-  if (threadIdx.x == 0) {
+  if (tid() == 0) {
     a.status[cell] = status;
     c.st->attempts = attempts;
     c.st->t_end_ns = (long long)globaltimer();
     if (a.stats) a.stats[cell] = *c.st;
   }
-  __syncthreads();
+  csync();
 }
 
 template <typename LT, bool GM, bool RK = false>
-__global__ void __launch_bounds__(NT, 1) solve_kernel(const SolveArgs a) {
+__global__ void __launch_bounds__(NT, CBX_CTAS) solve_kernel(const SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_cell;
   Smem s;
-  layout(a.net.S, a.net.R, a.net.nseg, sizeof(LT) == 4, GM, smem_raw, &s, a.piv_ints);
+  layout(a.net.S, a.net.R, a.net.nseg, sizeof(LT) == 4, GM, smem_raw, &s, a.piv_ints, CBX_LEAN);
   s.piv = global_pivots(a.net);
   if constexpr (!GM && sizeof(LT) == 8) {
     if (a.piv_ints > 0) stage_pivots(a.net, s);
   }
   double* ws = a.ws + (size_t)blockIdx.x * a.ws_stride;
+  if (CBX_LEAN) {
+    s.r = ws + a.net.R;  // where the Jacobian keeps its partials
+    s.part = s.r + a.net.R;
+  }
   for (;;) {
-    if (threadIdx.x == 0) s_cell = next_cell(a.counter, a.order, a.C);
-    __syncthreads();
+    if (tid() == 0) s_cell = next_cell(a.counter, a.order, a.C);
+    csync();
     const int cell = s_cell;
-    __syncthreads();
+    csync();
     if (cell < 0) break;
     if constexpr (RK)
       solve_cell_rk<LT, GM>(a, cell, s, ws);
