@@ -226,7 +226,7 @@ int cbx_network_symbolic(const cbx_network* net, int* perm, unsigned char* fill,
 
 static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double* x0, int C, double t0,
                       double t_end, const cbx_options* opt, void* stream, double* x_out, int* cell_status,
-                      cbx_cell_stats* stats, cbx_tape* tape, int max_grid = 0, const double* track = nullptr,
+                      cbx_cell_stats* stats, cbx_tape* tape, const LaunchLimits& limits = {}, const double* track = nullptr,
                       int K = 0, const double* alpha = nullptr, const double* t_end_cell = nullptr) {
   if (!net) return fail(CBX_E_ARG, "net is NULL");
   if (C < 0) return fail(CBX_E_ARG, "C must be >= 0");
@@ -244,7 +244,7 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (rc) return rc;
   const HostNet& h = net->host;
   const bool mixed = o.precision == CBX_MIXED;
-  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints);
+  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C);
   const int occ = plan.occupancy;
   if (occ < 1) {
     char m[200];
@@ -253,7 +253,8 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
     return fail(CBX_E_TOO_LARGE, m);
   }
   int grid = std::min(C, occ * device_sm_count());
-  if (max_grid > 0) grid = std::min(grid, max_grid);
+  if (limits.max_sms > 0) grid = std::min(grid, limits.max_sms * occ);
+  if (limits.max_ctas > 0) grid = std::min(grid, limits.max_ctas);
   cudaStream_t st = (cudaStream_t)stream;
   SolveArgs a{};
   a.net = net->dev;
@@ -283,7 +284,7 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (tape) a.tape = tape->dev;
   a.ws_stride = plan.ws_stride;
   // the cells' order follows the counter when some CTA takes a second cell
-  const bool ordered = C > grid;
+  const bool ordered = C > grid && limits.order;
   const size_t ws_bytes = (size_t)grid * a.ws_stride * sizeof(double) + 256 + (ordered ? (size_t)C * sizeof(int) : 0);
   void* ws = nullptr;
   cudaError_t e = cudaMallocAsync(&ws, ws_bytes, st);
@@ -355,7 +356,7 @@ int cbx_solve_track(cbx_network* net, const double* track, int K, const double* 
                     const cbx_options* opt, void* stream, double* x_out, int* cell_status, cbx_cell_stats* stats) {
   if (K < 1) return fail(CBX_E_ARG, "K must be >= 1");
   if (C > 0 && !track) return fail(CBX_E_ARG, "track is NULL");
-  return solve_impl(net, nullptr, x0, C, t0, t_end, opt, stream, x_out, cell_status, stats, nullptr, 0, track, K);
+  return solve_impl(net, nullptr, x0, C, t0, t_end, opt, stream, x_out, cell_status, stats, nullptr, {}, track, K);
 }
 
 int cbx_solve_host(cbx_network* net, const cbx_cell_params* phi, const double* x0, int C, double t0,
@@ -488,7 +489,7 @@ int cbx_solve_with_alpha(cbx_network* net, const double* alpha, const cbx_cell_p
     if (tape->net != net) return fail(CBX_E_ARG, "the tape belongs to another network");
     if (C > tape->C) return fail(CBX_E_ARG, "C exceeds the tape's capacity");
   }
-  return solve_impl(net, phi, x0, C, t0, t_end, opt, stream, x_out, cell_status, stats, tape, 0, nullptr, 0, alpha);
+  return solve_impl(net, phi, x0, C, t0, t_end, opt, stream, x_out, cell_status, stats, tape, {}, nullptr, 0, alpha);
 }
 
 int cbx_solve_track_record(cbx_network* net, const double* track, int K, const double* x0, int C, double t0,
@@ -499,7 +500,7 @@ int cbx_solve_track_record(cbx_network* net, const double* track, int K, const d
   if (C > tape->C) return fail(CBX_E_ARG, "C exceeds the tape's capacity");
   if (K < 1) return fail(CBX_E_ARG, "K must be >= 1");
   if (C > 0 && !track) return fail(CBX_E_ARG, "track is NULL");
-  return solve_impl(net, nullptr, x0, C, t0, t_end, opt, stream, x_out, cell_status, stats, tape, 0, track, K);
+  return solve_impl(net, nullptr, x0, C, t0, t_end, opt, stream, x_out, cell_status, stats, tape, {}, track, K);
 }
 
 int cbx_tape_step_times(const cbx_tape* tape, int cell, double* t_new, int cap) {
@@ -612,9 +613,9 @@ int cbx_tape_program(const cbx_tape* tape, int cell, int* kinds, int* qs, double
 
 namespace cbx {
 int solve_device(cbx_network* net, const cbx_cell_params* phi, const double* x0, int C, double t0, double t_end,
-                 const cbx_options* opt, void* stream, double* x_out, int* cell_status, int max_grid,
+                 const cbx_options* opt, void* stream, double* x_out, int* cell_status, const LaunchLimits& limits,
                  const double* t_end_cell) {
-  return solve_impl(net, phi, x0, C, t0, t_end, opt, stream, x_out, cell_status, nullptr, nullptr, max_grid, nullptr,
-                    0, nullptr, t_end_cell);
+  return solve_impl(net, phi, x0, C, t0, t_end, opt, stream, x_out, cell_status, nullptr, nullptr, limits, nullptr, 0,
+                    nullptr, t_end_cell);
 }
 }  // namespace cbx

@@ -182,16 +182,23 @@ int launch_env_grad(const double* gcell, int C, const DevNet& n, double* g_lnzet
 
 // Launch plan of the solver kernel for one network and precision: matrix in
 // shared memory (gm = false) or in the CTA's global workspace (gm = true).
+// CTA shapes of the solver kernel: 256 threads and an SM to themselves (the
+// fastest a single cell gets), or several CTAs (cells) per SM for batches.
+enum CtaShape { kOnePerSm = 0, kNarrow = 1, kMid = 2, kTwoPerSm = 3 };
+
 struct SolverPlan {
   bool mixed = false, gm = false;
   size_t smem = 0;          // dynamic shared memory per CTA
   long long ws_stride = 0;  // per-CTA global workspace, in doubles
   int occupancy = 0;        // CTAs per SM (0: cannot launch)
   int piv_ints = 0;         // staged pivot-list ints in shared memory (0: none)
+  CtaShape shape = kOnePerSm;
 };
 size_t smem_bytes(int S, int R, int nseg, bool mixed, bool gm, int piv_ints = 0);
 long long workspace_doubles(int S, int R, int nnzJ, bool mixed, bool gm);
-SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints);
+// The plan of a launch of C cells (its workspace per CTA does not depend on C,
+// and its occupancy is largest for the largest batches).
+SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C);
 // Launch the solver; returns a cudaError_t value.
 int launch_solver(const SolveArgs& a, const SolverPlan& p, int grid, void* stream);
 // One translation unit per kernel instantiation (precision x matrix placement).
@@ -203,6 +210,23 @@ int occupancy_solve_fp64(size_t smem);
 int occupancy_solve_fp64_gm(size_t smem);
 int occupancy_solve_mixed(size_t smem);
 int occupancy_solve_mixed_gm(size_t smem);
+// Shapes with several CTAs per SM: one translation unit holds both methods.
+int launch_solve_fp64_narrow(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_fp64_narrow(size_t smem);
+int launch_solve_fp64_mid(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_fp64_mid(size_t smem);
+int launch_solve_fp64_two(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_fp64_two(size_t smem);
+int launch_solve_fp64_gm_two(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_fp64_gm_two(size_t smem);
+int launch_solve_mixed_narrow(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_mixed_narrow(size_t smem);
+int launch_solve_mixed_mid(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_mixed_mid(size_t smem);
+int launch_solve_mixed_two(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_mixed_two(size_t smem);
+int launch_solve_mixed_gm_two(const SolveArgs& a, bool rk, size_t smem, int grid, void* stream);
+int occupancy_solve_mixed_gm_two(size_t smem);
 int launch_solve_fp64_rk(const SolveArgs& a, size_t smem, int grid, void* stream);
 int launch_solve_mixed_rk(const SolveArgs& a, size_t smem, int grid, void* stream);
 int launch_solve_fp64_gm_rk(const SolveArgs& a, size_t smem, int grid, void* stream);
@@ -210,11 +234,17 @@ int launch_solve_mixed_gm_rk(const SolveArgs& a, size_t smem, int grid, void* st
 // Launch the ESDIRK solver; returns a cudaError_t value.
 int launch_solver_rk(const SolveArgs& a, const SolverPlan& p, int grid, void* stream);
 int device_sm_count();
-// cbx_solve on device buffers with at most max_grid CTAs (0: no cap) and,
-// optionally, per-cell end times t_end_cell [C] (device; t_end must then be
-// their maximum).
+// What a launch may take of the device (0: no cap): the SMs' worth of CTAs, the
+// CTAs, and whether it has memory for the order of its cells.
+struct LaunchLimits {
+  int max_sms = 0;
+  int max_ctas = 0;
+  bool order = true;
+};
+// cbx_solve on device buffers within limits and, optionally, with per-cell end
+// times t_end_cell [C] (device; t_end must then be their maximum).
 int solve_device(cbx_network* net, const cbx_cell_params* phi, const double* x0, int C, double t0, double t_end,
-                 const cbx_options* opt, void* stream, double* x_out, int* cell_status, int max_grid,
+                 const cbx_options* opt, void* stream, double* x_out, int* cell_status, const LaunchLimits& limits,
                  const double* t_end_cell = nullptr);
 // Set the calling thread's cbx_last_error() message; returns code.
 int record_error(int code, const std::string& msg);

@@ -8,8 +8,8 @@
 // the launch's persistent CTAs back-fill across requests; a cell's solver
 // state stays on chip for its whole solve. Requests that arrive while others
 // run are admitted into the freed streams and memory, and their kernels run
-// concurrently with the running ones; each launch uses at most `max_ctas`
-// CTAs so that several launches, of any network size, share the SMs.
+// concurrently with the running ones; each launch uses at most `max_ctas` SMs'
+// worth of CTAs so that several launches, of any network size, share the SMs.
 //
 // Per launch: device buffers (inputs, outputs, per-cell end times, solver
 // workspace), the H2D copies of every merged request (strided copies into the
@@ -76,6 +76,7 @@ struct ServerRequest {
   // lock: the completion callback, on a driver thread, takes that lock)
   size_t cell_bytes = 0, cta_bytes = 0;
   int grid_cap = 1;
+  bool ordered = true;  // memory for the order of its cells is reserved
   double t_submit = 0, t_start = 0, t_done = 0;
 };
 
@@ -113,18 +114,19 @@ namespace {
 // so only outside the server's lock.
 void size_request(ServerRequest* r, int max_ctas) {
   const HostNet& h = r->net->host;
-  const SolverPlan p = plan_solver(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints);
+  const SolverPlan p = plan_solver(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints,
+                                   kMaxMergedCells);
   r->cell_bytes = sizeof(cbx_cell_params) + 2 * h.S * sizeof(double) + sizeof(double) + sizeof(int);
   r->cta_bytes = (size_t)p.ws_stride * sizeof(double);
-  r->grid_cap = std::max(1, std::max(1, p.occupancy) * device_sm_count());
-  if (max_ctas > 0) r->grid_cap = std::min(r->grid_cap, max_ctas);
+  const int occ = std::max(1, p.occupancy);  // of the largest batches: an upper bound
+  r->grid_cap = std::max(1, occ * (max_ctas > 0 ? std::min(max_ctas, device_sm_count()) : device_sm_count()));
 }
 
 // Device bytes of a launch of C cells of r's kind: inputs, outputs, end times,
 // status, workspace, order of the cells (pure arithmetic: safe under the lock).
 size_t launch_bytes(const ServerRequest* r, int C) {
   return (size_t)C * r->cell_bytes + (size_t)std::min(C, r->grid_cap) * r->cta_bytes +
-         (C > r->grid_cap ? (size_t)C * sizeof(int) : 0) + 8192;
+         (r->ordered && C > r->grid_cap ? (size_t)C * sizeof(int) : 0) + 8192;
 }
 
 bool same_kind(const ServerRequest* a, const ServerRequest* b) {
@@ -186,7 +188,8 @@ void launch(cbx_server* s, ServerLaunch* L) {
       o += r->C;
     }
     if (e == cudaSuccess) {
-      rc = solve_device(r0->net, d_phi, d_x0, C, r0->t0, t_max, &r0->opt, st, d_xo, d_st, s->max_ctas, d_t);
+      rc = solve_device(r0->net, d_phi, d_x0, C, r0->t0, t_max, &r0->opt, st, d_xo, d_st,
+                        LaunchLimits{s->max_ctas, r0->grid_cap, r0->ordered}, d_t);
       o = 0;
       for (ServerRequest* r : L->reqs) {
         if (rc == CBX_OK && e == cudaSuccess)
@@ -334,6 +337,13 @@ int cbx_server_submit(cbx_server* s, cbx_network* net, const cbx_cell_params* ph
   cbx_default_options(&r->opt);
   if (opt) r->opt = *opt;
   size_request(r, s->max_ctas);
+  if (launch_bytes(r, C) > s->budget) {
+    // a tight budget: as many CTAs as fit, in the cells' own order
+    r->ordered = false;
+    const size_t fixed = (size_t)C * r->cell_bytes + 8192;
+    const size_t fit = s->budget > fixed ? (s->budget - fixed) / std::max<size_t>(1, r->cta_bytes) : 0;
+    r->grid_cap = (int)std::min<size_t>(r->grid_cap, std::max<size_t>(1, fit));
+  }
   if (launch_bytes(r, C) > s->budget) {
     delete r;
     return record_error(CBX_E_TOO_LARGE, "request larger than the server's memory budget");
