@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const GradArgs a) {
           __syncthreads();
           const double c = v / a.gam[q];
           jacobian(n, kap, s.y, g, Jv);
-          build_matrix<double>(n, Jv, c, M);
+          build_matrix<double, false>(n, Jv, c, M);
           lu_crout64(global_pivots(n), M, invd);
           forwardT_crout64(M, S, s.dy);
           for (int i = threadIdx.x; i < S; i += NT) s.dy[i] *= invd[i];

@@ -12,7 +12,7 @@ size_t smem_bytes(int S, int R, int nseg, bool mixed, bool gm, int piv_ints) {
 long long workspace_doubles(int S, int R, int nnzJ, bool mixed, bool gm) {
   long long n = 3LL * R + nnzJ;
   n = (n + 31) / 32 * 32;
-  if (gm) n += ((long long)S * lead_dim(S) * (mixed ? 4 : 8) / 8 + 31) / 32 * 32;
+  if (gm) n += ((long long)S * lead_dim_gm(S) * (mixed ? 4 : 8) / 8 + 31) / 32 * 32;
   return n;
 }
 

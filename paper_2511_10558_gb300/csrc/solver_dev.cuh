@@ -334,9 +334,15 @@ __device__ void jacobian(const DevNet& n, const double* __restrict__ kap, const 
 
 __host__ __device__ inline int lead_dim(int S) { return S | 1; }  // odd: conflict-free column access
 
-template <typename LT>
+// Leading dimension of a matrix in global memory: rows start on 16 bytes (one
+// thread's 32 entries of a row are 16-byte loads), an odd number of 16-byte
+// (FP32) or 32-byte (FP64) units apart, so that a column's rows spread over the
+// cache's sets.
+__host__ __device__ inline int lead_dim_gm(int S) { return 4 * (((S + 3) / 4) | 1); }
+
+template <typename LT, bool GM>
 __device__ void build_matrix(const DevNet& n, const double* Jv, double c, LT* M) {
-  const int S = n.S, ld = lead_dim(S);
+  const int S = n.S, ld = GM ? lead_dim_gm(S) : lead_dim(S);
   for (int idx = tid(); idx < S * ld; idx += NT) M[idx] = LT(0);
   csync();
   for (int s = tid(); s < n.nnzJ; s += NT) {
@@ -981,15 +987,52 @@ constexpr int NB = 32;  // panel width
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
-template <typename LT, bool FULL, int RPT>
+// One thread's NB entries of a row, in 16-byte pieces: of a matrix in global
+// memory (lead_dim_gm, columns from a multiple of NB on). A warp's scalar load
+// touches 32 rows' lines for 4 or 8 bytes of each, and the cache takes a line a
+// cycle; 16 bytes at a time need a quarter (FP32) or half (FP64) of those.
+__device__ __forceinline__ void load_row(const float* p, float (&r)[NB]) {
+#pragma unroll
+  for (int c = 0; c < NB; c += 4) {
+    const float4 q = *(const float4*)(p + c);
+    r[c] = q.x, r[c + 1] = q.y, r[c + 2] = q.z, r[c + 3] = q.w;
+  }
+}
+__device__ __forceinline__ void load_row(const double* p, double (&r)[NB]) {
+#pragma unroll
+  for (int c = 0; c < NB; c += 2) {
+    const double2 q = *(const double2*)(p + c);
+    r[c] = q.x, r[c + 1] = q.y;
+  }
+}
+__device__ __forceinline__ void store_row(float* p, const float (&r)[NB]) {
+#pragma unroll
+  for (int c = 0; c < NB; c += 4) *(float4*)(p + c) = make_float4(r[c], r[c + 1], r[c + 2], r[c + 3]);
+}
+__device__ __forceinline__ void store_row(double* p, const double (&r)[NB]) {
+#pragma unroll
+  for (int c = 0; c < NB; c += 2) *(double2*)(p + c) = make_double2(r[c], r[c + 1]);
+}
+
+// VEC: the matrix is in global memory (16-byte rows).
+template <typename LT, bool FULL, int RPT, bool VEC>
 __device__ __forceinline__ void panel_factor(LT* M, LT* invd, int S, int ld, int kb, int nb) {
   const int t = tid();
   LT r[RPT][NB];
 #pragma unroll
   for (int p = 0; p < RPT; ++p) {
     const int i = kb + t + NT * p;
+    if constexpr (FULL && VEC) {
+      if (i < S) {
+        load_row(M + i * ld + kb, r[p]);
+      } else {  // (left undefined, these made the kernel spill 7 KB)
 #pragma unroll
-    for (int jj = 0; jj < NB; ++jj) r[p][jj] = i < S && (FULL || jj < nb) ? M[i * ld + kb + jj] : LT(0);
+        for (int jj = 0; jj < NB; ++jj) r[p][jj] = LT(0);
+      }
+    } else {
+#pragma unroll
+      for (int jj = 0; jj < NB; ++jj) r[p][jj] = i < S && (FULL || jj < nb) ? M[i * ld + kb + jj] : LT(0);
+    }
   }
 #pragma unroll
   for (int c = 0; c < NB; ++c) {
@@ -1023,9 +1066,13 @@ __device__ __forceinline__ void panel_factor(LT* M, LT* invd, int S, int ld, int
     const int i = kb + t + NT * p;
     if (i >= S) continue;
     if (i >= kb + nb) {
+      if constexpr (FULL && VEC) {
+        store_row(M + i * ld + kb, r[p]);
+      } else {
 #pragma unroll
-      for (int jj = 0; jj < NB; ++jj)
-        if (FULL || jj < nb) M[i * ld + kb + jj] = r[p][jj];
+        for (int jj = 0; jj < NB; ++jj)
+          if (FULL || jj < nb) M[i * ld + kb + jj] = r[p][jj];
+      }
     } else {
       // rows of the diagonal block: only their L part (columns < own row) is new
 #pragma unroll
@@ -1367,37 +1414,32 @@ __device__ void invert_upper_blocks(LT* M, const LT* invd, int S, int ld) {
 }
 
 // A22 -= L21 U12 for one of the leading panels [kb, kb+NB) of a network whose
-// first pivots are sparse: one thread per trailing row i; for each pivot k of
-// the panel with L(i,k) != 0, the columns j >= kb+NB of U(k,:) from the
-// pivot's structural list (ascending). Rows are disjoint, so no two threads
-// write one element. Entries outside the pattern hold exact zeros, so the
-// skipped terms are exact zeros.
+// first pivots are sparse: a warp takes a trailing row i; for each pivot k of
+// the panel with L(i,k) != 0, its lanes take the columns j >= kb+NB of U(k,:)
+// from the pivot's structural list. Rows are disjoint, so no two warps write
+// one element, and an element's terms come in pivot order. Entries outside the
+// pattern hold exact zeros, so the skipped terms are exact zeros. (A thread per
+// row walked the list with a line of its own for each access: 500 species FP64,
+// 160 cells to 1e3 yr 509 ms, so 489 ms.)
 template <typename LT>
 __device__ void sparse_panel_update(LT* M, int S, int ld, int kb, const int* uptr, const int* ucol) {
   const int ke = kb + NB;
-  for (int i = ke + tid(); i < S; i += NT) {
+  const int warp = tid() >> 5, lane = tid() & 31;
+  for (int i = ke + warp; i < S; i += NW) {
     LT* row = M + (size_t)i * ld;
-    for (int c = 0; c < NB; ++c) {
-      const LT l = row[kb + c];
-      if (l == LT(0)) continue;
-      const int k = kb + c;
+    const LT lv = row[kb + lane];
+    unsigned left = __ballot_sync(FULL, lv != LT(0));
+    while (left) {
+      const int c = __ffs(left) - 1, k = kb + c;
+      left &= left - 1;
+      const LT l = __shfl_sync(FULL, lv, c);
       const LT* urow = M + (size_t)k * ld;
       const int e1 = uptr[k + 1];
-      int e = uptr[k];
-      while (e < e1 && ucol[e] < ke) ++e;  // columns inside the panel
-      for (; e + 4 <= e1; e += 4) {
-        const int j0 = ucol[e], j1 = ucol[e + 1], j2 = ucol[e + 2], j3 = ucol[e + 3];
-        const LT u0 = urow[j0], u1 = urow[j1], u2 = urow[j2], u3 = urow[j3];
-        const LT a0 = row[j0], a1 = row[j1], a2 = row[j2], a3 = row[j3];
-        row[j0] = a0 - l * u0;
-        row[j1] = a1 - l * u1;
-        row[j2] = a2 - l * u2;
-        row[j3] = a3 - l * u3;
-      }
-      for (; e < e1; ++e) {
+      for (int e = uptr[k] + lane; e < e1; e += 32) {
         const int j = ucol[e];
-        row[j] -= l * urow[j];
+        if (j >= ke) row[j] -= l * urow[j];
       }
+      __syncwarp();  // the next pivot's lanes may take other columns
     }
   }
   csync();
@@ -1417,8 +1459,8 @@ __device__ void sparse_panel_update(LT* M, int S, int ld, int kb, const int* upt
 #endif
 
 __device__ __forceinline__ void panel_factor_full_rows(float* M, float* invd, int S, int ld, int kb) {
-  if (S - kb > NT) panel_factor<float, true, 2>(M, invd, S, ld, kb, NB);
-  else panel_factor<float, true, 1>(M, invd, S, ld, kb, NB);
+  if (S - kb > NT) panel_factor<float, true, 2, true>(M, invd, S, ld, kb, NB);
+  else panel_factor<float, true, 1, true>(M, invd, S, ld, kb, NB);
 }
 
 __device__ __noinline__ void lu_blocked_pairs(float* M, float* invd, int S, int ld) {
@@ -1441,7 +1483,7 @@ __device__ __noinline__ void lu_blocked_pairs(float* M, float* invd, int S, int 
       panel_factor_full_rows(M, invd, S, ld, kb);
       panel_u12<float, true>(M, S, ld, kb, nb);
     } else {
-      panel_factor<float, false, 1>(M, invd, S, ld, kb, nb);
+      panel_factor<float, false, 1, true>(M, invd, S, ld, kb, nb);
       panel_u12<float, false>(M, S, ld, kb, nb);
     }
     tc_rect<4>(M, ld, kb, nb, kb + nb, S, kb + nb, S);
@@ -1469,17 +1511,31 @@ __device__ void lu_blocked(LT* M, LT* invd, int S, int ld, int nsp = 0, const in
     const int nb = min(NB, S - kb);
     const bool two = LARGE && S - kb > NT;  // more panel rows than threads
     if (nb == NB) {
-      if (two) panel_factor<LT, true, LARGE ? 2 : 1>(M, invd, S, ld, kb, nb);
-      else panel_factor<LT, true, 1>(M, invd, S, ld, kb, nb);
+      if (two) panel_factor<LT, true, LARGE ? 2 : 1, LARGE>(M, invd, S, ld, kb, nb);
+      else panel_factor<LT, true, 1, LARGE>(M, invd, S, ld, kb, nb);
       panel_u12<LT, true>(M, S, ld, kb, nb);
     } else {
-      panel_factor<LT, false, 1>(M, invd, S, ld, kb, nb);
+      panel_factor<LT, false, 1, LARGE>(M, invd, S, ld, kb, nb);
       panel_u12<LT, false>(M, S, ld, kb, nb);
     }
     if (LARGE && sizeof(LT) == 8 && kb < nsp * NB) sparse_panel_update<LT>(M, S, ld, kb, uptr, ucol);
     else trailing_update<LT, LARGE>(M, S, ld, kb, nb);
   }
   invert_upper_blocks<LT>(M, invd, S, ld);
+}
+
+// v - sum_c m[c] vb[c] of one row, four partial sums
+template <typename LT, bool FULL>
+__device__ __forceinline__ LT row_minus_block(const LT (&m)[NB], const LT* vb, int nb, LT v) {
+  LT p0 = v, p1 = LT(0), p2 = LT(0), p3 = LT(0);
+#pragma unroll
+  for (int c = 0; c < NB; c += 4) {
+    if (FULL || c < nb) p0 -= m[c] * vb[c];
+    if (FULL || c + 1 < nb) p1 -= m[c + 1] * vb[c + 1];
+    if (FULL || c + 2 < nb) p2 -= m[c + 2] * vb[c + 2];
+    if (FULL || c + 3 < nb) p3 -= m[c + 3] * vb[c + 3];
+  }
+  return (p0 + p1) + (p2 + p3);
 }
 
 template <typename LT, bool FULL>
@@ -1499,51 +1555,74 @@ __device__ __forceinline__ void rows_minus_block(const LT* M, int ld, const LT* 
   }
 }
 
-template <typename LT>
+// The diagonal block's product with its stored inverse (warp 0): lane i of the
+// block takes row i; UPPER: U_bb^{-1} (its diagonal in invd), else L_bb^{-1}.
+template <typename LT, bool VEC, bool UPPER>
+__device__ __forceinline__ void block_product(const LT* M, const LT* invd, int ld, int kb, int nb, LT* v, int lane) {
+  LT acc = LT(0);
+  const LT* row = M + (kb + min(lane, nb - 1)) * ld + kb;
+  if (VEC && nb == NB) {
+    LT m[NB];
+    load_row(row, m);
+    acc = UPPER ? invd[kb + lane] * v[kb + lane] : v[kb + lane];
+#pragma unroll
+    for (int c = UPPER ? 1 : 0; c < (UPPER ? NB : NB - 1); ++c)
+      if (UPPER ? c > lane : c < lane) acc += m[c] * v[kb + c];
+  } else if (lane < nb) {
+    acc = UPPER ? invd[kb + lane] * v[kb + lane] : v[kb + lane];
+#pragma unroll
+    for (int c = UPPER ? 1 : 0; c < (UPPER ? NB : NB - 1); ++c)
+      if (UPPER ? c > lane && c < nb : c < lane) acc += row[c] * v[kb + c];
+  }
+  __syncwarp();
+  if (lane < nb) v[kb + lane] = acc;
+}
+
+// v <- U^{-1} L^{-1} v with the inverted diagonal blocks, block by block. VEC:
+// the matrix is in global memory, where a block's step costs the latency and
+// the cache lines of its loads: they are 16 bytes wide, and each thread has its
+// first row's on the way before the barrier behind which the block's values
+// are. With the panel's rows read and written the same way: 500 species mixed,
+// 200 cells to 1e4 yr 262 -> 237 ms, 333 species 231 -> 188 ms.
+template <typename LT, bool VEC>
 __device__ void solve_blocked(const LT* M, const LT* invd, int S, int ld, LT* v) {
   const int warp = tid() >> 5, lane = tid() & 31;
-  for (int kb = 0; kb < S; kb += NB) {
-    const int nb = min(NB, S - kb), ke = kb + nb;
-    if (warp == 0) {
-      LT acc = LT(0);
-      const LT* row = M + (kb + min(lane, nb - 1)) * ld + kb;
-      if (lane < nb) {
-        acc = v[kb + lane];
-#pragma unroll
-        for (int c = 0; c < NB - 1; ++c)
-          if (c < lane) acc += row[c] * v[kb + c];
+  auto rows = [&](int kb, int nb, int i0, int i1, auto diag) {
+    if (VEC && nb == NB) {
+      LT m[NB];
+      const int i = i0 + tid();
+      if (i < i1) load_row(M + i * ld + kb, m);
+      if (warp == 0) diag();
+      csync();
+      if (i < i1) v[i] = row_minus_block<LT, true>(m, v + kb, nb, v[i]);
+      for (int i2 = i + NT; i2 < i1; i2 += NT) {
+        load_row(M + i2 * ld + kb, m);
+        v[i2] = row_minus_block<LT, true>(m, v + kb, nb, v[i2]);
       }
-      __syncwarp();
-      if (lane < nb) v[kb + lane] = acc;
+    } else {
+      if (warp == 0) diag();
+      csync();
+      if (nb == NB)
+        rows_minus_block<LT, true>(M + kb, ld, v + kb, nb, v, i0, i1);
+      else
+        rows_minus_block<LT, false>(M + kb, ld, v + kb, nb, v, i0, i1);
     }
     csync();
-    if (nb == NB)
-      rows_minus_block<LT, true>(M + kb, ld, v + kb, nb, v, ke, S);
-    else
-      rows_minus_block<LT, false>(M + kb, ld, v + kb, nb, v, ke, S);
-    csync();
+  };
+  for (int kb = 0; kb < S; kb += NB) {
+    const int nb = min(NB, S - kb);
+    rows(kb, nb, kb + nb, S, [&] { block_product<LT, VEC, false>(M, invd, ld, kb, nb, v, lane); });
   }
   for (int kb = ((S - 1) / NB) * NB; kb >= 0; kb -= NB) {
     const int nb = min(NB, S - kb);
-    if (warp == 0) {
-      LT acc = LT(0);
-      const LT* row = M + (kb + min(lane, nb - 1)) * ld + kb;
-      if (lane < nb) {
-        acc = invd[kb + lane] * v[kb + lane];
-#pragma unroll
-        for (int c = 1; c < NB; ++c)
-          if (c > lane && c < nb) acc += row[c] * v[kb + c];
-      }
-      __syncwarp();
-      if (lane < nb) v[kb + lane] = acc;
-    }
-    csync();
-    if (nb == NB)
-      rows_minus_block<LT, true>(M + kb, ld, v + kb, nb, v, 0, kb);
-    else
-      rows_minus_block<LT, false>(M + kb, ld, v + kb, nb, v, 0, kb);
-    csync();
+    rows(kb, nb, 0, kb, [&] { block_product<LT, VEC, true>(M, invd, ld, kb, nb, v, lane); });
   }
+}
+
+// Not inlined: as with lu_blocked_pairs, the kernel body spills otherwise.
+template <typename LT>
+__device__ __noinline__ void solve_blocked_gm(const LT* M, const LT* invd, int S, LT* v) {
+  solve_blocked<LT, true>(M, invd, S, lead_dim_gm(S), v);
 }
 
 // ---------------------------------------------------------------- shared layout
@@ -1726,7 +1805,7 @@ template <bool GM>
 __device__ void linear_solve(Cell<double, GM>& c, double cc, const double* w, double* dy) {
   const int S = c.n.S;
   if constexpr (GM) {
-    solve_blocked<double>(c.M, (const double*)c.s.invd, S, lead_dim(S), dy);
+    solve_blocked_gm<double>(c.M, (const double*)c.s.invd, S, dy);
   } else {
     forward_crout64(c.M, (const double*)c.s.invd, S, dy, c.s.red);
     backward_crout64(c.M, S, dy, c.s.red);
@@ -1742,8 +1821,11 @@ __device__ void linear_solve(Cell<float, GM>& c, double cc, const double* w, dou
   const float* M = c.M;
   const float* invd = (const float*)c.s.invd;
   float* v = c.s.v32;
-  const int ld = lead_dim(S);
-  solve_blocked<float>(M, invd, S, ld, v);
+  auto solve = [&] {
+    if constexpr (GM) solve_blocked_gm<float>(M, invd, S, v);
+    else solve_blocked<float, false>(M, invd, S, lead_dim(S), v);
+  };
+  solve();
   for (int i = tid(); i < S; i += NT) dy[i] = (double)v[i];
   csync();
   for (int sweep = 0; sweep < c.a.max_refine; ++sweep) {
@@ -1755,7 +1837,7 @@ __device__ void linear_solve(Cell<float, GM>& c, double cc, const double* w, dou
       v[i] = (float)res;
     }
     csync();
-    solve_blocked<float>(M, invd, S, ld, v);
+    solve();
     double* slot = c.s.sc.next();
     chunk_sums(
         [&](int i) {
@@ -1779,9 +1861,9 @@ __device__ void linear_solve(Cell<float, GM>& c, double cc, const double* w, dou
 
 template <typename LT, bool GM>
 __device__ void factor(Cell<LT, GM>& c, double cc) {
-  build_matrix<LT>(c.n, c.Jv, cc, c.M);
+  build_matrix<LT, GM>(c.n, c.Jv, cc, c.M);
   if constexpr (GM) {
-    lu_blocked<LT, true>(c.M, (LT*)c.s.invd, c.n.S, lead_dim(c.n.S), c.n.sparse_panels, c.n.piv_uptr, c.n.piv_u);
+    lu_blocked<LT, true>(c.M, (LT*)c.s.invd, c.n.S, lead_dim_gm(c.n.S), c.n.sparse_panels, c.n.piv_uptr, c.n.piv_u);
   } else {
     if constexpr (sizeof(LT) == 4)
       lu_blocked<LT, false>(c.M, (LT*)c.s.invd, c.n.S, lead_dim(c.n.S));
