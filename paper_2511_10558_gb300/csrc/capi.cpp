@@ -62,7 +62,7 @@ int upload(cbx_network* n) {
          o_gamma = pk.add(h.gamma), o_ra = pk.add(h.ra), o_rb = pk.add(h.rb), o_seg = pk.add(h.seg_ptr),
          o_sps = pk.add(h.spec_seg), o_ent = pk.add(h.rhs_ent), o_jrow = pk.add(h.jrow),
          o_jcol = pk.add(h.jcol), o_jrp = pk.add(h.jrow_ptr), o_jgp = pk.add(h.jg_ptr),
-         o_jgs = pk.add(h.jg_slot), o_jgl = pk.add(h.jg_len), o_jgt = pk.add(h.jg_term), o_plp = pk.add(h.piv_lptr), o_pl = pk.add(h.piv_l),
+         o_jgs = pk.add(h.jg_slot), o_jgl = pk.add(h.jg_len), o_jgt = pk.add(h.jg_term), o_pe = pk.add(h.piv_end), o_plp = pk.add(h.piv_lptr), o_pl = pk.add(h.piv_l),
          o_pup = pk.add(h.piv_uptr), o_pu = pk.add(h.piv_u), o_perm = pk.add(h.perm),
          o_rprod = pk.add(h.rprod), o_rj = pk.add(h.rj), o_gb = pk.add(h.gbeta), o_gg = pk.add(h.ggamma);
   cudaGetDevice(&n->device);
@@ -102,6 +102,7 @@ int upload(cbx_network* n) {
   d.jg_slot = (const int*)(b + o_jgs);
   d.jg_len = (const int*)(b + o_jgl);
   d.jg_term = (const int*)(b + o_jgt);
+  d.piv_end = (const int*)(b + o_pe);
   d.piv_lptr = (const int*)(b + o_plp);
   d.piv_l = (const int*)(b + o_pl);
   d.piv_uptr = (const int*)(b + o_pup);

@@ -44,6 +44,7 @@ struct DevNet {
   const int* piv_l;
   const int* piv_uptr;   // [S+1] range of columns j > k with U(k,j) structurally non-zero
   const int* piv_u;
+  const int* piv_end;    // [kdense] end of the run of independent pivots that holds k
   const int* perm;       // [S] internal -> user species index
   const int* rprod;      // [4R] products of each reaction (internal), -1 absent
   // Reactions grouped by rate type, so that each type's rate coefficients are
@@ -72,7 +73,7 @@ enum { kOpInit = 0, kOpRescale = 1, kOpStep = 2 };
 // Host-side compiled network.
 struct HostNet {
   int S = 0, R = 0, nnzJ = 0, nnzLU = 0, nseg = 0, kdense = 0;
-  int head_ints = 0;  // 2 (kdense + 1) + entries of the sparse pivots' lists
+  int head_ints = 0;  // 2 (kdense + 1) + kdense + entries of the sparse pivots' lists
   int sparse_panels = 0;  // see DevNet
   double lu_flops = 0;
   std::vector<int> perm, iperm, rprod;
@@ -82,7 +83,7 @@ struct HostNet {
   std::vector<int> jrow, jcol, jrow_ptr;
   int njg = 0;
   std::vector<int> jg_ptr, jg_slot, jg_len, jg_term;
-  std::vector<int> piv_lptr, piv_l, piv_uptr, piv_u;
+  std::vector<int> piv_end, piv_lptr, piv_l, piv_uptr, piv_u;
   int tptr[kNumTypes + 1] = {};
   std::vector<int> rj;
   std::vector<double> gbeta, ggamma;

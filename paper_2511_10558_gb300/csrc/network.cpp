@@ -288,7 +288,19 @@ std::string compile_network(const cbx_species* sp, int S, const cbx_reaction* rx
       }
     }
   }
-  n.head_ints = 2 * (n.kdense + 1) + n.piv_lptr[n.kdense] + n.piv_uptr[n.kdense];
+  // Runs of sparse pivots none of which is in another's row or column: their U
+  // rows are prepared side by side and their updates share two barriers.
+  for (int k = 0; k < n.kdense;) {
+    int e = k + 1;
+    auto apart = [&](int m) {
+      for (int p = k; p < m; ++p)
+        if (F[(size_t)m * S + p] || F[(size_t)p * S + m]) return false;
+      return true;
+    };
+    while (e < n.kdense && apart(e)) ++e;
+    for (; k < e; ++k) n.piv_end.push_back(e);
+  }
+  n.head_ints = 2 * (n.kdense + 1) + n.kdense + n.piv_lptr[n.kdense] + n.piv_uptr[n.kdense];
   // Leading 32-wide panels of the FP64 blocked LU (networks whose matrix lives
   // in global memory) whose trailing update is applied from the pivot lists
   // rather than as a dense rank-32 product: a panel counts while the

@@ -374,10 +374,11 @@ struct PivLists {
   const int* l;
   const int* uptr;  // [kd+1]
   const int* u;
+  const int* end;   // [kd] end of the run of independent pivots that holds k
 };
 
 __device__ __forceinline__ PivLists global_pivots(const DevNet& n) {
-  return PivLists{n.S, n.kdense, n.piv_lptr, n.piv_l, n.piv_uptr, n.piv_u};
+  return PivLists{n.S, n.kdense, n.piv_lptr, n.piv_l, n.piv_uptr, n.piv_u, n.piv_end};
 }
 
 __device__ __forceinline__ int lrow(const PivLists& P, bool dense, int k, int e) {
@@ -477,6 +478,70 @@ __device__ __forceinline__ void crout_rows(const PivLists& P, double* M, double*
     double* r1 = two ? M + lrow(P, dense, k, e + nw) * ld : r0;
     update_rows<MC>(r0, r1, two, k, jc, uv, nu, lane);
   }
+}
+
+// Sparse pivot k of a run of independent ones: row i of L(:,k) belongs to warp
+// i mod NW for every pivot of the run, so that a row takes the run's pivots in
+// order without a barrier.
+template <int MC>
+__device__ __forceinline__ void run_rows(const PivLists& P, double* M, int k, int u0, int nu) {
+  const int ld = lead_dim(P.S);
+  const int w = tid() >> 5, lane = tid() & 31;
+  int jc[MC];
+  double uv[MC];
+#pragma unroll
+  for (int m = 0; m < MC; ++m) {
+    const int b = lane + 32 * m;
+    jc[m] = b < nu ? P.u[u0 + b] : 0;
+    uv[m] = b < nu ? M[k * ld + jc[m]] : 0.0;
+  }
+  const int l1 = P.lptr[k + 1];
+  for (int l0 = P.lptr[k]; l0 < l1; l0 += 32) {
+    const int i = l0 + lane < l1 ? P.l[l0 + lane] : 0;
+    unsigned mine = __ballot_sync(FULL, l0 + lane < l1 && i % NW == w);
+    while (mine) {
+      const int i0 = __shfl_sync(FULL, i, __ffs(mine) - 1);
+      mine &= mine - 1;
+      const bool two = mine != 0;
+      const int i1 = two ? __shfl_sync(FULL, i, __ffs(mine) - 1) : i0;
+      if (two) mine &= mine - 1;
+      update_rows<MC>(M + i0 * ld, M + i1 * ld, two, k, jc, uv, nu, lane);
+    }
+  }
+  __syncwarp();  // the next pivot's lanes may take other columns
+}
+
+// Where the SM holds three or more cells (fewer threads each) the others fill
+// such waits and rows dealt by number are less even than rows dealt in turn: 61
+// species, 1,000 cells 98 ms with single pivots, 100 ms with runs.
+constexpr bool kRuns = NT == 256;
+
+// Pivots k .. end-1, independent of one another (none in another's row or
+// column): their U rows are prepared a warp each (row k is ready if said so),
+// then all rows take their updates. Two barriers a run where single pivots take
+// one each, and behind each of those waited for warp 0's reciprocal and scaling:
+// 150 species has 23 sparse pivots in runs of 10, 7, 3 and 3. 150 species, 1,216
+// cells to 1 Myr 393 -> 385 ms; 97 species ESDIRK 218 -> 215 ms; one cell of 32
+// species 13.7 -> 13.3 ms.
+__device__ void crout_run(const PivLists& P, double* M, double* invd, int k, int end, bool ready) {
+  const int w = tid() >> 5, lane = tid() & 31;
+  for (int m = k + (ready ? 1 : 0) + w; m < end; m += NW) prep_pivot(P, M, invd, m, lane);
+  csync();
+  for (int m = k; m < end; ++m) {
+    const int u0 = P.uptr[m], nu = P.uptr[m + 1] - u0;
+    switch ((nu + 31) >> 5) {
+      case 0: break;
+      case 1: run_rows<1>(P, M, m, u0, nu); break;
+      case 2: if constexpr (kMaxColRegs >= 2) run_rows<2>(P, M, m, u0, nu); break;
+      case 3: if constexpr (kMaxColRegs >= 3) run_rows<3>(P, M, m, u0, nu); break;
+      case 4: if constexpr (kMaxColRegs >= 4) run_rows<4>(P, M, m, u0, nu); break;
+      case 5: if constexpr (kMaxColRegs >= 5) run_rows<5>(P, M, m, u0, nu); break;
+      case 6: if constexpr (kMaxColRegs >= 6) run_rows<6>(P, M, m, u0, nu); break;
+      case 7: if constexpr (kMaxColRegs >= 7) run_rows<7>(P, M, m, u0, nu); break;
+      default: if constexpr (kMaxColRegs >= 8) run_rows<8>(P, M, m, u0, nu); break;
+    }
+  }
+  csync();
 }
 
 // Dense range, first step: pivot k alone brings rows k+1 and k+2 to final (U
@@ -753,8 +818,22 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
   const int kp = max(kd, S - 1 - DENSE_PAIR_COLS);
   const bool pairs = S - kp >= 3;
   const int k_single = pairs ? kp : S - 1;
-  for (int k = 0; k < k_single; ++k) {
+  bool ready = true;  // U row k is prepared
+  int k = 0;
+  for (; k < k_single; ++k) {
     const bool dense = k >= kd;
+    if (kRuns && !dense && P.end[k] > k + 1) {
+      const int end = P.end[k];
+      crout_run(P, M, invd, k, end, ready);
+      ready = false;
+      k = end - 1;
+      continue;
+    }
+    if (!ready) {
+      if (w == 0) prep_pivot(P, M, invd, k, lane);
+      csync();
+      ready = true;
+    }
     int l0, l1, u0, nu;
     if (dense) {
       l0 = 0;
@@ -783,6 +862,10 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
     } else if (w == 0 && next_in_l) {
       prep_pivot(P, M, invd, k + 1, lane);
     }
+    csync();
+  }
+  if (!ready && k < S) {  // a run ended just before the pairs or the last pivot
+    if (w == 0) prep_pivot(P, M, invd, k, lane);
     csync();
   }
   if (pairs) {
@@ -1685,16 +1768,18 @@ __device__ void stage_pivots(const DevNet& n, Smem& s) {
   const int nl = n.piv_lptr[kd], nu = n.piv_uptr[kd];
   int* lp = s.pstage;
   int* up = lp + (kd + 1);
-  int* l = up + (kd + 1);
+  int* end = up + (kd + 1);
+  int* l = end + kd;
   int* u = l + nl;
   for (int i = tid(); i <= kd; i += NT) {
     lp[i] = n.piv_lptr[i];
     up[i] = n.piv_uptr[i];
   }
+  for (int i = tid(); i < kd; i += NT) end[i] = n.piv_end[i];
   for (int i = tid(); i < nl; i += NT) l[i] = n.piv_l[i];
   for (int i = tid(); i < nu; i += NT) u[i] = n.piv_u[i];
   csync();
-  s.piv = PivLists{n.S, kd, lp, l, up, u};
+  s.piv = PivLists{n.S, kd, lp, l, up, u, end};
 }
 
 
