@@ -1497,30 +1497,56 @@ __device__ void invert_upper_blocks(LT* M, const LT* invd, int S, int ld) {
 }
 
 // A22 -= L21 U12 for one of the leading panels [kb, kb+NB) of a network whose
-// first pivots are sparse: a warp takes a trailing row i; for each pivot k of
-// the panel with L(i,k) != 0, its lanes take the columns j >= kb+NB of U(k,:)
-// from the pivot's structural list. Rows are disjoint, so no two warps write
-// one element, and an element's terms come in pivot order. Entries outside the
-// pattern hold exact zeros, so the skipped terms are exact zeros. (A thread per
-// row walked the list with a line of its own for each access: 500 species FP64,
-// 160 cells to 1e3 yr 509 ms, so 489 ms.)
+// first pivots are sparse: eight lanes take a trailing row i; for each pivot k
+// of the panel with L(i,k) != 0 they take the columns j >= kb+NB of U(k,:) from
+// the pivot's structural list, 32 at a time. Rows are disjoint, so no two warps
+// write one element, and an element's terms come in pivot order. Entries outside
+// the pattern hold exact zeros, so the skipped terms are exact zeros. Bound by
+// the latency of list, then values, in global memory: a row has two or three
+// such pivots of 30 to 50 columns, so lanes go to many rows at once. 500 species,
+// cycles a panel: a thread a row 2.3 M (a cache line of its own for each access),
+// a warp a row 1.8 M, this 1.5 M.
 template <typename LT>
 __device__ void sparse_panel_update(LT* M, int S, int ld, int kb, const int* uptr, const int* ucol) {
   const int ke = kb + NB;
-  const int warp = tid() >> 5, lane = tid() & 31;
-  for (int i = ke + warp; i < S; i += NW) {
-    LT* row = M + (size_t)i * ld;
-    const LT lv = row[kb + lane];
-    unsigned left = __ballot_sync(FULL, lv != LT(0));
-    while (left) {
-      const int c = __ffs(left) - 1, k = kb + c;
-      left &= left - 1;
-      const LT l = __shfl_sync(FULL, lv, c);
-      const LT* urow = M + (size_t)k * ld;
-      const int e1 = uptr[k + 1];
-      for (int e = uptr[k] + lane; e < e1; e += 32) {
-        const int j = ucol[e];
-        if (j >= ke) row[j] -= l * urow[j];
+  const int lane = tid() & 31, l8 = lane & 7;
+  for (int i0 = ke; i0 < S; i0 += NT / 8) {  // (the same number of passes for every lane of a warp)
+    const int i = i0 + (tid() >> 3);
+    LT* row = M + (size_t)min(i, S - 1) * ld;
+    LT lv[4];
+    unsigned left = 0;  // the pivots of this row
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      lv[m] = i < S ? row[kb + l8 + 8 * m] : LT(0);
+      left |= (__ballot_sync(FULL, lv[m] != LT(0)) >> (lane & 24) & 0xffu) << (8 * m);
+    }
+    while (__any_sync(FULL, left != 0)) {
+      const int c = left ? __ffs(left) - 1 : 0;
+      LT l = LT(0);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const LT lm = __shfl_sync(FULL, lv[m], c & 7, 8);
+        if (c >> 3 == m) l = lm;
+      }
+      if (left) {
+        const int k = kb + c;
+        const LT* urow = M + (size_t)k * ld;
+        const int e1 = uptr[k + 1];
+        for (int e = uptr[k] + l8; e < e1; e += 32) {
+          int j[4];
+          LT u[4], x[4];
+#pragma unroll
+          for (int m = 0; m < 4; ++m) j[m] = e + 8 * m < e1 ? ucol[e + 8 * m] : 0;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            u[m] = j[m] >= ke ? urow[j[m]] : LT(0);
+            x[m] = j[m] >= ke ? row[j[m]] : LT(0);
+          }
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+            if (j[m] >= ke) row[j[m]] = x[m] - l * u[m];
+        }
+        left &= left - 1;
       }
       __syncwarp();  // the next pivot's lanes may take other columns
     }
