@@ -1692,7 +1692,8 @@ __device__ __forceinline__ void block_product(const LT* M, const LT* invd, int l
 // the cache lines of its loads: they are 16 bytes wide, and each thread has its
 // first row's on the way before the barrier behind which the block's values
 // are. With the panel's rows read and written the same way: 500 species mixed,
-// 200 cells to 1e4 yr 262 -> 237 ms, 333 species 231 -> 188 ms.
+// 200 cells to 1e4 yr 262 -> 190 ms, 333 species 231 -> 160 ms. (In shared memory
+// the early loads cost more than they save: 150 species mixed 233 -> 247 ms.)
 template <typename LT, bool VEC>
 __device__ void solve_blocked(const LT* M, const LT* invd, int S, int ld, LT* v) {
   const int warp = tid() >> 5, lane = tid() & 31;
@@ -1700,7 +1701,12 @@ __device__ void solve_blocked(const LT* M, const LT* invd, int S, int ld, LT* v)
     if (VEC && nb == NB) {
       LT m[NB];
       const int i = i0 + tid();
-      if (i < i1) load_row(M + i * ld + kb, m);
+      if (i < i1) {
+        load_row(M + i * ld + kb, m);
+      } else {  // (left undefined, these made the function spill all of them)
+#pragma unroll
+        for (int c = 0; c < NB; ++c) m[c] = LT(0);
+      }
       if (warp == 0) diag();
       csync();
       if (i < i1) v[i] = row_minus_block<LT, true>(m, v + kb, nb, v[i]);
