@@ -314,14 +314,14 @@ int grad_occupancy(int S, int R, int nseg) {
   const size_t sm = smem_bytes(S, R, nseg, false, false);
   if (S > 32 * kMaxColRegs || sm > device_smem_optin()) return 0;
   int blocks = 0;
-  cudaError_t e = cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = open_shared_memory(grad_kernel);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, grad_kernel, NT, sm);
   return e == cudaSuccess ? blocks : 0;
 }
 
 int launch_grad(const GradArgs& a, int grid, void* stream) {
   const size_t sm = smem_bytes(a.net.S, a.net.R, a.net.nseg, false, false);
-  cudaError_t e = cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const cudaError_t e = open_shared_memory(grad_kernel);
   if (e != cudaSuccess) return e;
   grad_kernel<<<grid, NT, sm, (cudaStream_t)stream>>>(a);
   return cudaGetLastError();

@@ -2509,9 +2509,23 @@ __global__ void __launch_bounds__(NT, CBX_CTAS) solve_kernel(const SolveArgs a) 
   }
 }
 
+// Opens a kernel to all the dynamic shared memory a CTA can have. Networks of
+// every size share a kernel, and a thread may plan a small one between another
+// thread's call here and its launch: the limit has to be the same in all calls
+// (it was each network's own size, and such a launch failed). The launch's own
+// size sets what it takes of the SM.
+template <typename K>
+static cudaError_t open_shared_memory(K* kernel) {
+  cudaFuncAttributes f;
+  const cudaError_t e = cudaFuncGetAttributes(&f, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(device_smem_optin() - f.sharedSizeBytes));
+}
+
 template <typename LT, bool GM, bool RK = false>
 static int launch_t(const SolveArgs& a, size_t sm, int grid, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(solve_kernel<LT, GM, RK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const cudaError_t e = open_shared_memory(solve_kernel<LT, GM, RK>);
   if (e != cudaSuccess) return e;
   solve_kernel<LT, GM, RK><<<grid, NT, sm, st>>>(a);
   return cudaGetLastError();
@@ -2520,7 +2534,7 @@ static int launch_t(const SolveArgs& a, size_t sm, int grid, cudaStream_t st) {
 template <typename LT, bool GM>
 static int occupancy_t(size_t sm) {
   int blocks = 0;
-  cudaError_t e = cudaFuncSetAttribute(solve_kernel<LT, GM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = open_shared_memory(solve_kernel<LT, GM>);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, solve_kernel<LT, GM>, NT, sm);
   return e == cudaSuccess ? blocks : 0;
 }
