@@ -47,7 +47,7 @@ ShapeKernel shape_kernel(const SolverPlan& p) {
 SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C) {
   SolverPlan p;
   p.mixed = mixed;
-  const size_t optin = device_smem_optin();
+  const size_t optin = device_smem_optin() - kStaticShared;
   // shared-memory matrix when it fits and the FP64 LU's register tiling allows (S <= 256)
   p.gm = !(S <= 32 * kMaxColRegs && smem_bytes(S, R, nseg, mixed, false) <= optin);
   p.smem = smem_bytes(S, R, nseg, mixed, p.gm);

@@ -1752,6 +1752,10 @@ struct Smem {
   PivLists piv;  // the lists the LU reads
 };
 
+// Static shared memory of the solver kernels (s_cell, s_stats): a CTA's dynamic
+// part can be the device's limit less this.
+constexpr size_t kStaticShared = 8 + sizeof(cbx_cell_stats);
+
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
 // Lean: the rates r and the segment sums part live in the CTA's workspace (they
