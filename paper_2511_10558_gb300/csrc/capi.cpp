@@ -245,17 +245,14 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (rc) return rc;
   const HostNet& h = net->host;
   const bool mixed = o.precision == CBX_MIXED;
-  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C);
-  const int occ = plan.occupancy;
-  if (occ < 1) {
+  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C, limits.max_ctas);
+  if (plan.occupancy < 1) {
     char m[200];
     snprintf(m, sizeof m, "network (S=%d, R=%d) needs %zu B of shared memory per CTA (S <= %d); the device allows %zu",
              h.S, h.R, plan.smem, 512, device_smem_optin());
     return fail(CBX_E_TOO_LARGE, m);
   }
-  int grid = std::min(C, occ * device_sm_count());
-  if (limits.max_sms > 0) grid = std::min(grid, limits.max_sms * occ);
-  if (limits.max_ctas > 0) grid = std::min(grid, limits.max_ctas);
+  const int grid = launch_grid(plan, C, limits.max_ctas);
   cudaStream_t st = (cudaStream_t)stream;
   SolveArgs a{};
   a.net = net->dev;

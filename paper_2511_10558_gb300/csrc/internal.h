@@ -193,13 +193,22 @@ struct SolverPlan {
   long long ws_stride = 0;  // per-CTA global workspace, in doubles
   int occupancy = 0;        // CTAs per SM (0: cannot launch)
   int piv_ints = 0;         // staged pivot-list ints in shared memory (0: none)
+  int sms = 0;              // of the device
   CtaShape shape = kOnePerSm;
+};
+// What the plan of a launch is chosen from.
+struct LaunchForms {
+  int S = 0, R = 0, nseg = 0;
+  size_t lean = 0;     // dynamic shared memory per CTA of the lean layout
+  SolverPlan form[4];  // by CtaShape, with their occupancies
 };
 size_t smem_bytes(int S, int R, int nseg, bool mixed, bool gm, int piv_ints = 0);
 long long workspace_doubles(int S, int R, int nnzJ, bool mixed, bool gm);
-// The plan of a launch of C cells (its workspace per CTA does not depend on C,
-// and its occupancy is largest for the largest batches).
-SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C);
+// The plan of a launch of C cells with at most max_ctas CTAs (0: no limit). Its
+// workspace per CTA depends on neither.
+SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C, int max_ctas);
+// The CTAs of that launch.
+int launch_grid(const SolverPlan& p, int C, int max_ctas);
 // Launch the solver; returns a cudaError_t value.
 int launch_solver(const SolveArgs& a, const SolverPlan& p, int grid, void* stream);
 // One translation unit per kernel instantiation (precision x matrix placement).
@@ -235,10 +244,9 @@ int launch_solve_mixed_gm_rk(const SolveArgs& a, size_t smem, int grid, void* st
 // Launch the ESDIRK solver; returns a cudaError_t value.
 int launch_solver_rk(const SolveArgs& a, const SolverPlan& p, int grid, void* stream);
 int device_sm_count();
-// What a launch may take of the device (0: no cap): the SMs' worth of CTAs, the
-// CTAs, and whether it has memory for the order of its cells.
+// What a launch may take of the device: its CTAs (0: no cap), and whether it has
+// memory for the order of its cells.
 struct LaunchLimits {
-  int max_sms = 0;
   int max_ctas = 0;
   bool order = true;
 };

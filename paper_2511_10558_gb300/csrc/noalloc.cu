@@ -117,10 +117,7 @@ extern "C" int cbx_solve_noalloc(cbx_network* net, const cbx_cell_params* phi, c
   }
   const HostNet& h = net->host;
   const bool mixed = o.precision == CBX_MIXED;
-  auto plan_for = [&](long long cells) {
-    return plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, (int)std::min<long long>(C, cells));
-  };
-  const SolverPlan one = plan_for(1);
+  const SolverPlan one = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, 1, 0);
   if (one.occupancy < 1) return fail(CBX_E_TOO_LARGE, "network too large for the solver");
   const long long stride = one.ws_stride;
   const long long fit = (long long)((kScratchBytes - kCounterBytes) / (stride * sizeof(double)));
@@ -130,10 +127,9 @@ extern "C" int cbx_solve_noalloc(cbx_network* net, const cbx_cell_params* phi, c
              (long long)(stride * sizeof(double)), kScratchBytes - kCounterBytes);
     return fail(CBX_E_TOO_LARGE, m);
   }
-  // the shape for the cells that the array lets run at a time, if it limits them
-  const SolverPlan plan = plan_for(fit < device_sm_count() ? fit : C);
-  const int occ = plan.occupancy;
-  const int grid = (int)std::min<long long>(std::min<long long>(C, (long long)occ * device_sm_count()), fit);
+  const int max_ctas = (int)std::min<long long>(fit, C);
+  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C, max_ctas);
+  const int grid = launch_grid(plan, C, max_ctas);
   SolveArgs a{};
   a.net = net->dev;
   a.alpha = net->dev.alpha;

@@ -1,6 +1,8 @@
 // Launch planning of the solver kernel (host code): shared-memory and
 // workspace sizes, the matrix placement, occupancy, and the dispatch to the
 // translation unit holding each kernel instantiation.
+#include <algorithm>
+
 #include "solver_dev.cuh"
 
 namespace cbx {
@@ -42,11 +44,64 @@ ShapeKernel shape_kernel(const SolverPlan& p) {
                  : ShapeKernel{launch_solve_fp64_two, occupancy_solve_fp64_two};
 }
 
-}  // namespace
+// Whether the network can take a shape with several CTAs on an SM: the most
+// species that its kernels hold, and the shared memory of its CTAs.
+bool takes(const LaunchForms& f, CtaShape shape) {
+  const SolverPlan& one = f.form[kOnePerSm];
+  auto fits = [&](size_t smem, int ctas) { return (smem + kCtaReserved) * ctas <= kSmShared; };
+  if (shape == kNarrow) return !one.gm && f.S <= 48 && fits(one.smem, 5);
+  if (f.nseg > f.R) return false;  // no room for the segment sums in the lean layout
+  if (shape == kMid) return !one.gm && f.S <= 96 && fits(f.lean, 3);
+  return (one.gm || f.S <= (one.mixed ? 160 : 128)) && fits(f.lean, 2);
+}
 
-SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C) {
-  SolverPlan p;
+// Batches: several cells per SM. A cell is slower beside others (they share
+// the FP64 pipe) but leaves the SM fewer idle cycles, so a shape pays once the
+// batch is bound by throughput rather than by its costliest cell; the more
+// of a cell's time is serial (small networks), the sooner. Measured with
+// cells of 1e5 yr (500 species: 1e3 yr), times in ms by cells:
+//   32 species:  160/304/608/1216 cells, one per SM 17/24/41/77, mid
+//                13/13/16/30, narrow 15/14/16/22
+//   61:          one 57/67/127/227, two 60/64/95/163, mid 64/66/72/125
+//   80:          one 39/58/93/169, two 37/51/70/117, mid 40/57/67/102
+//   97:          one 92/80/121/224, two 99/92/93/167 (mixed, 304/608/1216:
+//                one 77/115/215, two 83/84/148)
+//   150 mixed:   one 81/84/86/174, two 92/104/119/130
+//   500 mixed:   160/304/608 cells, one 137/210/365, two 150/181/292;
+//   500 FP64:    304 cells, one 743, two 647; 200 FP64: 304/608 cells, one
+//                210/355, two 214/270
+CtaShape batch_shape(const LaunchForms& f, int C) {
+  const SolverPlan& one = f.form[kOnePerSm];
+  const double load = (double)C / one.sms;  // cells per SM
+  if (one.gm) return load >= (f.S > 256 ? 2.0 : 4.0) && takes(f, kTwoPerSm) ? kTwoPerSm : kOnePerSm;
+  if (load >= 6.0 && takes(f, kNarrow)) return kNarrow;
+  if (load > (f.S <= 48 ? 1.0 : 4.0) && takes(f, kMid)) return kMid;
+  if (load >= (f.S <= 96 ? 1.5 : one.mixed && f.S > 112 ? 6.0 : 4.0) && takes(f, kTwoPerSm)) return kTwoPerSm;
+  return kOnePerSm;
+}
+
+// The plan of a shape with several CTAs on an SM, or that of one cell to an SM
+// where the device would not run more CTAs of it.
+void query_form(LaunchForms& f, CtaShape shape) {
+  const SolverPlan& one = f.form[kOnePerSm];
+  SolverPlan p = one;
+  p.shape = shape;
+  if (shape != kNarrow) {
+    p.smem = f.lean;
+    p.piv_ints = 0;
+  }
+  p.occupancy = shape_kernel(p).occupancy(p.smem);
+  f.form[shape] = p.occupancy > one.occupancy ? p : one;
+}
+
+LaunchForms base_form(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints) {
+  LaunchForms f;
+  f.S = S;
+  f.R = R;
+  f.nseg = nseg;
+  SolverPlan& p = f.form[kOnePerSm];
   p.mixed = mixed;
+  p.sms = device_sm_count();
   const size_t optin = device_smem_optin() - kStaticShared;
   // shared-memory matrix when it fits and the FP64 LU's register tiling allows (S <= 256)
   p.gm = !(S <= 32 * kMaxColRegs && smem_bytes(S, R, nseg, mixed, false) <= optin);
@@ -58,51 +113,39 @@ SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_in
   }
   p.ws_stride = workspace_doubles(S, R, nnzJ, mixed, p.gm);
   p.occupancy = 0;
-  if (S > 2 * NT || p.smem > optin) return p;
+  if (S > 2 * NT || p.smem > optin) return f;
   if (mixed)
     p.occupancy = p.gm ? occupancy_solve_mixed_gm(p.smem) : occupancy_solve_mixed(p.smem);
   else
     p.occupancy = p.gm ? occupancy_solve_fp64_gm(p.smem) : occupancy_solve_fp64(p.smem);
-  if (p.occupancy < 1) return p;
-  // Batches: several cells per SM. A cell is slower beside others (they share
-  // the FP64 pipe) but leaves the SM fewer idle cycles, so a shape pays once the
-  // batch is bound by throughput rather than by its costliest cell; the more
-  // of a cell's time is serial (small networks), the sooner. Measured with
-  // cells of 1e5 yr (500 species: 1e3 yr), times in ms by cells:
-  //   32 species:  160/304/608/1216 cells, one per SM 17/24/41/77, mid
-  //                13/13/16/30, narrow 15/14/16/22
-  //   61:          one 57/67/127/227, two 60/64/95/163, mid 64/66/72/125
-  //   80:          one 39/58/93/169, two 37/51/70/117, mid 40/57/67/102
-  //   97:          one 92/80/121/224, two 99/92/93/167 (mixed, 304/608/1216:
-  //                one 77/115/215, two 83/84/148)
-  //   150 mixed:   one 81/84/86/174, two 92/104/119/130
-  //   500 mixed:   160/304/608 cells, one 137/210/365, two 150/181/292;
-  //   500 FP64:    304 cells, one 743, two 647; 200 FP64: 304/608 cells, one
-  //                210/355, two 214/270
-  const double load = (double)C / device_sm_count();  // cells per SM
-  const bool lean_ok = nseg <= R;
-  const size_t full = p.smem, lean = layout(S, R, nseg, mixed, p.gm, nullptr, nullptr, 0, true);
-  auto fits = [&](size_t smem, int ctas) { return (smem + kCtaReserved) * ctas <= kSmShared; };
-  CtaShape shape = kOnePerSm;
-  if (p.gm) {
-    if (load >= (S > 256 ? 2.0 : 4.0) && lean_ok && fits(lean, 2)) shape = kTwoPerSm;
-  } else if (S <= 48 && load >= 6.0 && fits(full, 5)) {
-    shape = kNarrow;
-  } else if (S <= 96 && load > (S <= 48 ? 1.0 : 4.0) && lean_ok && fits(lean, 3)) {
-    shape = kMid;
-  } else if (S <= (mixed ? 160 : 128) && load >= (S <= 96 ? 1.5 : mixed && S > 112 ? 6.0 : 4.0) && lean_ok &&
-             fits(lean, 2)) {
-    shape = kTwoPerSm;
-  }
-  if (shape == kOnePerSm) return p;
-  SolverPlan b = p;
-  b.shape = shape;
-  if (shape != kNarrow) {
-    b.smem = lean;
-    b.piv_ints = 0;
-  }
-  b.occupancy = shape_kernel(b).occupancy(b.smem);
-  return b.occupancy > p.occupancy ? b : p;
+  f.lean = layout(S, R, nseg, mixed, p.gm, nullptr, nullptr, 0, true);
+  return f;
+}
+
+template <typename Form>
+SolverPlan choose(const LaunchForms& f, int C, int max_ctas, Form form) {
+  if (max_ctas > 0 && max_ctas <= f.form[kOnePerSm].sms) return f.form[kOnePerSm];
+  const SolverPlan p = form(batch_shape(f, C));
+  // A limit that leaves less than half of the shape's CTAs: the shape for as many
+  // cells as it lets run at a time (48 species, 150 CTAs: narrow 23 ms, one to an
+  // SM 15; 150 species mixed, 204 of 304 CTAs: two to an SM 126, one 130).
+  return max_ctas > 0 && max_ctas < launch_grid(p, C, 0) / 2 ? form(batch_shape(f, max_ctas)) : p;
+}
+
+}  // namespace
+
+SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C, int max_ctas) {
+  LaunchForms f = base_form(S, R, nseg, nnzJ, mixed, head_ints);
+  if (f.form[kOnePerSm].occupancy < 1) return f.form[kOnePerSm];
+  return choose(f, C, max_ctas, [&](CtaShape s) {
+    if (s != kOnePerSm) query_form(f, s);
+    return f.form[s];
+  });
+}
+
+int launch_grid(const SolverPlan& p, int C, int max_ctas) {
+  const int grid = std::min(C, p.occupancy * p.sms);
+  return max_ctas > 0 ? std::min(grid, max_ctas) : grid;
 }
 
 int launch_solver(const SolveArgs& a0, const SolverPlan& p, int grid, void* stream) {

@@ -8,8 +8,8 @@
 // the launch's persistent CTAs back-fill across requests; a cell's solver
 // state stays on chip for its whole solve. Requests that arrive while others
 // run are admitted into the freed streams and memory, and their kernels run
-// concurrently with the running ones; each launch uses at most `max_ctas` SMs'
-// worth of CTAs so that several launches, of any network size, share the SMs.
+// concurrently with the running ones; each launch uses at most `max_ctas` CTAs
+// so that several launches, of any network size, share the SMs.
 //
 // Per launch: device buffers (inputs, outputs, per-cell end times, solver
 // workspace), the H2D copies of every merged request (strided copies into the
@@ -115,11 +115,12 @@ namespace {
 void size_request(ServerRequest* r, int max_ctas) {
   const HostNet& h = r->net->host;
   const SolverPlan p = plan_solver(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints,
-                                   kMaxMergedCells);
+                                   kMaxMergedCells, 0);
   r->cell_bytes = sizeof(cbx_cell_params) + 2 * h.S * sizeof(double) + sizeof(double) + sizeof(int);
   r->cta_bytes = (size_t)p.ws_stride * sizeof(double);
   const int occ = std::max(1, p.occupancy);  // of the largest batches: an upper bound
-  r->grid_cap = std::max(1, occ * (max_ctas > 0 ? std::min(max_ctas, device_sm_count()) : device_sm_count()));
+  r->grid_cap = std::max(1, occ * device_sm_count());
+  if (max_ctas > 0) r->grid_cap = std::min(r->grid_cap, max_ctas);
 }
 
 // Device bytes of a launch of C cells of r's kind: inputs, outputs, end times,
@@ -189,7 +190,7 @@ void launch(cbx_server* s, ServerLaunch* L) {
     }
     if (e == cudaSuccess) {
       rc = solve_device(r0->net, d_phi, d_x0, C, r0->t0, t_max, &r0->opt, st, d_xo, d_st,
-                        LaunchLimits{s->max_ctas, r0->grid_cap, r0->ordered}, d_t);
+                        LaunchLimits{r0->grid_cap, r0->ordered}, d_t);
       o = 0;
       for (ServerRequest* r : L->reqs) {
         if (rc == CBX_OK && e == cudaSuccess)
