@@ -207,6 +207,10 @@ long long workspace_doubles(int S, int R, int nnzJ, bool mixed, bool gm);
 // The plan of a launch of C cells with at most max_ctas CTAs (0: no limit). Its
 // workspace per CTA depends on neither.
 SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C, int max_ctas);
+// The same without a CUDA call at the choice: the forms, for launches of up to
+// max_ctas CTAs (0: no limit), and the plan from them.
+LaunchForms launch_forms(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int max_ctas);
+SolverPlan choose_form(const LaunchForms& f, int C, int max_ctas);
 // The CTAs of that launch.
 int launch_grid(const SolverPlan& p, int C, int max_ctas);
 // Launch the solver; returns a cudaError_t value.

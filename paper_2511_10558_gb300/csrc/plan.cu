@@ -134,6 +134,21 @@ SolverPlan choose(const LaunchForms& f, int C, int max_ctas, Form form) {
 
 }  // namespace
 
+LaunchForms launch_forms(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int max_ctas) {
+  LaunchForms f = base_form(S, R, nseg, nnzJ, mixed, head_ints);
+  const SolverPlan& one = f.form[kOnePerSm];
+  if (one.occupancy < 1) return f;
+  for (CtaShape shape : {kNarrow, kMid, kTwoPerSm}) {
+    if ((max_ctas == 0 || max_ctas > one.sms) && takes(f, shape)) query_form(f, shape);
+    else f.form[shape] = one;
+  }
+  return f;
+}
+
+SolverPlan choose_form(const LaunchForms& f, int C, int max_ctas) {
+  return choose(f, C, max_ctas, [&](CtaShape s) { return f.form[s]; });
+}
+
 SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C, int max_ctas) {
   LaunchForms f = base_form(S, R, nseg, nnzJ, mixed, head_ints);
   if (f.form[kOnePerSm].occupancy < 1) return f.form[kOnePerSm];

@@ -75,8 +75,8 @@ struct ServerRequest {
   // launch sizing, computed at submit (no CUDA call may run under the server's
   // lock: the completion callback, on a driver thread, takes that lock)
   size_t cell_bytes = 0, cta_bytes = 0;
-  int grid_cap = 1;
-  bool ordered = true;  // memory for the order of its cells is reserved
+  LaunchForms forms;
+  LaunchLimits least;  // one cell to an SM, in the callers' order: the least workspace
   double t_submit = 0, t_start = 0, t_done = 0;
 };
 
@@ -85,6 +85,7 @@ struct ServerLaunch {
   cbx_server* srv = nullptr;
   std::vector<ServerRequest*> reqs;
   int C = 0;
+  LaunchLimits limits;
   size_t bytes = 0;
   int stream = -1;
 };
@@ -114,20 +115,22 @@ namespace {
 // so only outside the server's lock.
 void size_request(ServerRequest* r, int max_ctas) {
   const HostNet& h = r->net->host;
-  const SolverPlan p = plan_solver(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints,
-                                   kMaxMergedCells, 0);
+  r->forms = launch_forms(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints, max_ctas);
+  const SolverPlan& one = r->forms.form[kOnePerSm];
   r->cell_bytes = sizeof(cbx_cell_params) + 2 * h.S * sizeof(double) + sizeof(double) + sizeof(int);
-  r->cta_bytes = (size_t)p.ws_stride * sizeof(double);
-  const int occ = std::max(1, p.occupancy);  // of the largest batches: an upper bound
-  r->grid_cap = std::max(1, occ * device_sm_count());
-  if (max_ctas > 0) r->grid_cap = std::min(r->grid_cap, max_ctas);
+  r->cta_bytes = (size_t)one.ws_stride * sizeof(double);
+  r->least.max_ctas = std::max(1, one.occupancy) * one.sms;
+  if (max_ctas > 0) r->least.max_ctas = std::min(r->least.max_ctas, max_ctas);
+  r->least.order = false;
 }
 
-// Device bytes of a launch of C cells of r's kind: inputs, outputs, end times,
-// status, workspace, order of the cells (pure arithmetic: safe under the lock).
-size_t launch_bytes(const ServerRequest* r, int C) {
-  return (size_t)C * r->cell_bytes + (size_t)std::min(C, r->grid_cap) * r->cta_bytes +
-         (r->ordered && C > r->grid_cap ? (size_t)C * sizeof(int) : 0) + 8192;
+// Device bytes of a launch of C cells of r's kind within limits: inputs, outputs,
+// end times, status, workspace, order of the cells (pure arithmetic: safe under
+// the lock).
+size_t launch_bytes(const ServerRequest* r, int C, const LaunchLimits& limits) {
+  const int grid = std::max(1, launch_grid(choose_form(r->forms, C, limits.max_ctas), C, limits.max_ctas));
+  return (size_t)C * r->cell_bytes + grid * r->cta_bytes + (limits.order && C > grid ? (size_t)C * sizeof(int) : 0) +
+         8192;
 }
 
 bool same_kind(const ServerRequest* a, const ServerRequest* b) {
@@ -189,8 +192,7 @@ void launch(cbx_server* s, ServerLaunch* L) {
       o += r->C;
     }
     if (e == cudaSuccess) {
-      rc = solve_device(r0->net, d_phi, d_x0, C, r0->t0, t_max, &r0->opt, st, d_xo, d_st,
-                        LaunchLimits{r0->grid_cap, r0->ordered}, d_t);
+      rc = solve_device(r0->net, d_phi, d_x0, C, r0->t0, t_max, &r0->opt, st, d_xo, d_st, L->limits, d_t);
       o = 0;
       for (ServerRequest* r : L->reqs) {
         if (rc == CBX_OK && e == cudaSuccess)
@@ -216,12 +218,17 @@ void launch(cbx_server* s, ServerLaunch* L) {
 
 // Pick the next launch from the queue (lock held): the first request that
 // fits, unless an earlier one has been passed too often, plus the queued
-// requests of the same kind that fit with it. Returns null when nothing fits.
+// requests of the same kind that fit with it. What fits is judged by the least
+// that a launch takes; a launch gets the plan of its size (more CTAs of small
+// networks, the cells' order) where that keeps no other waiting: it costs at
+// most an eighth of the memory that the queued requests leave, and as many
+// launches of this size fit beside it as without. Returns null when nothing
+// fits.
 ServerLaunch* next_launch(cbx_server* s) {
   auto fits = [&](size_t bytes) { return s->in_use + bytes <= s->budget || s->in_use == 0; };
   ServerRequest* head = nullptr;
   for (ServerRequest* r : s->queue) {
-    if (fits(launch_bytes(r, r->C))) {
+    if (fits(launch_bytes(r, r->C, r->least))) {
       head = r;
       break;
     }
@@ -233,13 +240,15 @@ ServerLaunch* next_launch(cbx_server* s) {
   for (ServerRequest* r : s->queue) {
     if (r != head && !(same_kind(r, head) && L->C > 0)) continue;
     // a merged launch must fit the budget itself (the head alone always may run on an idle server)
-    if (r == head || (L->C + r->C <= kMaxMergedCells && s->in_use + launch_bytes(head, L->C + r->C) <= s->budget)) {
+    if (r == head || (L->C + r->C <= kMaxMergedCells &&
+                      s->in_use + launch_bytes(head, L->C + r->C, head->least) <= s->budget)) {
       L->reqs.push_back(r);
       L->C += r->C;
     }
   }
   // head first in the launch: requests merged before it in arrival order were skipped above
-  L->bytes = launch_bytes(head, L->C);
+  L->limits = head->least;
+  L->bytes = launch_bytes(head, L->C, L->limits);
   for (ServerRequest* r : s->queue) {
     if (r == head) break;
     if (std::find(L->reqs.begin(), L->reqs.end(), r) == L->reqs.end()) r->passed++;
@@ -248,6 +257,17 @@ ServerLaunch* next_launch(cbx_server* s) {
   for (ServerRequest* r : s->queue)
     if (std::find(L->reqs.begin(), L->reqs.end(), r) == L->reqs.end()) rest.push_back(r);
   s->queue.swap(rest);
+  size_t taken = s->in_use + L->bytes;
+  for (ServerRequest* r : s->queue) taken += launch_bytes(r, r->C, r->least);
+  const LaunchLimits full{s->max_ctas, true};
+  const size_t bytes = launch_bytes(head, L->C, full), extra = bytes - L->bytes;
+  const size_t left = taken <= s->budget ? s->budget - taken : 0;
+  const size_t streams = std::count(s->busy.begin(), s->busy.end(), 0) - 1;  // free beside this launch's
+  auto beside = [&](size_t room) { return std::min(streams, room / L->bytes); };
+  if (extra <= left / 8 && beside(left - extra) == beside(left)) {
+    L->limits = full;
+    L->bytes = bytes;
+  }
   return L;
 }
 
@@ -338,14 +358,7 @@ int cbx_server_submit(cbx_server* s, cbx_network* net, const cbx_cell_params* ph
   cbx_default_options(&r->opt);
   if (opt) r->opt = *opt;
   size_request(r, s->max_ctas);
-  if (launch_bytes(r, C) > s->budget) {
-    // a tight budget: as many CTAs as fit, in the cells' own order
-    r->ordered = false;
-    const size_t fixed = (size_t)C * r->cell_bytes + 8192;
-    const size_t fit = s->budget > fixed ? (s->budget - fixed) / std::max<size_t>(1, r->cta_bytes) : 0;
-    r->grid_cap = (int)std::min<size_t>(r->grid_cap, std::max<size_t>(1, fit));
-  }
-  if (launch_bytes(r, C) > s->budget) {
+  if (launch_bytes(r, C, r->least) > s->budget) {
     delete r;
     return record_error(CBX_E_TOO_LARGE, "request larger than the server's memory budget");
   }
