@@ -245,14 +245,17 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (rc) return rc;
   const HostNet& h = net->host;
   const bool mixed = o.precision == CBX_MIXED;
-  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C, limits.max_ctas);
+  auto plan_for = [&](int cells, int max_ctas) {
+    return plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, cells, max_ctas);
+  };
+  SolverPlan plan = plan_for(C, limits.max_ctas);
   if (plan.occupancy < 1) {
     char m[200];
     snprintf(m, sizeof m, "network (S=%d, R=%d) needs %zu B of shared memory per CTA (S <= %d); the device allows %zu",
              h.S, h.R, plan.smem, 512, device_smem_optin());
     return fail(CBX_E_TOO_LARGE, m);
   }
-  const int grid = launch_grid(plan, C, limits.max_ctas);
+  int grid = launch_grid(plan, C, limits.max_ctas);
   cudaStream_t st = (cudaStream_t)stream;
   SolveArgs a{};
   a.net = net->dev;
@@ -282,10 +285,20 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (tape) a.tape = tape->dev;
   a.ws_stride = plan.ws_stride;
   // the cells' order follows the counter when some CTA takes a second cell
-  const bool ordered = C > grid && limits.order;
-  const size_t ws_bytes = (size_t)grid * a.ws_stride * sizeof(double) + 256 + (ordered ? (size_t)C * sizeof(int) : 0);
+  bool ordered = C > grid && limits.order;
+  auto ws_bytes = [&] {
+    return (size_t)grid * a.ws_stride * sizeof(double) + 256 + (ordered ? (size_t)C * sizeof(int) : 0);
+  };
   void* ws = nullptr;
-  cudaError_t e = cudaMallocAsync(&ws, ws_bytes, st);
+  cudaError_t e = cudaMallocAsync(&ws, ws_bytes(), st);
+  if (e == cudaErrorMemoryAllocation && (plan.shape != kOnePerSm || ordered)) {
+    // no memory for several cells to an SM or for the order: the least workspace
+    cudaGetLastError();
+    plan = plan_for(1, 0);
+    grid = launch_grid(plan, C, limits.max_ctas);
+    ordered = false;
+    e = cudaMallocAsync(&ws, ws_bytes(), st);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(workspace)");
   a.ws = (double*)ws;
   a.counter = (int*)((char*)ws + (size_t)grid * a.ws_stride * sizeof(double));
