@@ -58,24 +58,47 @@ bool takes(const LaunchForms& f, CtaShape shape) {
 // Batches: several cells per SM. A cell is slower beside others (they share
 // the FP64 pipe) but leaves the SM fewer idle cycles, so a shape pays once the
 // batch is bound by throughput rather than by its costliest cell; the more
-// of a cell's time is serial (small networks), the sooner. Measured with
-// cells of 1e5 yr (500 species: 1e3 yr), times in ms by cells:
-//   32 species:  160/304/608/1216 cells, one per SM 17/24/41/77, mid
-//                13/13/16/30, narrow 15/14/16/22
-//   61:          one 57/67/127/227, two 60/64/95/163, mid 64/66/72/125
-//   80:          one 39/58/93/169, two 37/51/70/117, mid 40/57/67/102
-//   97:          one 92/80/121/224, two 99/92/93/167 (mixed, 304/608/1216:
-//                one 77/115/215, two 83/84/148)
-//   150 mixed:   one 81/84/86/174, two 92/104/119/130
-//   500 mixed:   160/304/608 cells, one 137/210/365, two 150/181/292;
-//   500 FP64:    304 cells, one 743, two 647; 200 FP64: 304/608 cells, one
-//                210/355, two 214/270
+// of a cell's time is serial (small networks), the sooner. Measured on one GB300
+// (152 SMs), ms, medians of five calls (which differ by 2 to 10 %, by up to 20 %
+// where few cells end a launch), by cells; BDF, 32 to 80 species 1e5 yr, 96 to
+// 200 1e4, 500 1e3:
+//               cells      153   200   304   456   608   912  1216  2432
+//   32 FP64     one         14    20    24          42    59    77   144
+//               mid         13    13    14          16    25    30    52
+//               narrow      14    14    15          16    19    22    42
+//   48 FP64     one         15    19    23          41    58    76   147
+//               mid         17    16    18          22    30    36    66
+//               narrow      23    22    24          26    33    39    63
+//   61 FP64     one         53    66    68    98   126   157   210
+//               two         56    60    58    77    92   117   149
+//               mid         62    61    62    68    78   103   123
+//   80 mixed    one         36          62    84   103   147   191
+//               two         36          47    60    75   102   130
+//               mid         37          47    59    67    86   111
+//   96 FP64     one         33          44    58    71   100   130
+//               two         35          48    53    56    74    95
+//   97 FP64     one         35          58    69    89   128   167
+//               two         37          67    56    67    93   120
+//   150 mixed   one         53          60          64    79   105 (1501: 131)
+//               two         62          75          90    89    86 (1501: 100)
+//   200 FP64    one        143         182   254   327
+//               two        151         219   241   277
+//   500 mixed   one         95         153   212   269
+//               two        113         148   180   227
+//   500 FP64    one        442         696   929
+//               two        479         663   860
+// The line moves with the span, as the costliest cells' share does: 150 mixed, 912
+// cells over 1e2 and 1e6 yr, one 48 and 175, two 37 and 146; 500 mixed, 304 cells
+// over 1e4 yr, one 218, two 268. The ESDIRK's solves are more of its
+// time, which moves it too; just above one cell an SM, at 45 to 48 species, mid
+// was slower with it than one to an SM (153 cells of 48: 53 against 49 ms; 160: 41
+// against 38), so mid begins there at 1.1.
 CtaShape batch_shape(const LaunchForms& f, int C) {
   const SolverPlan& one = f.form[kOnePerSm];
   const double load = (double)C / one.sms;  // cells per SM
   if (one.gm) return load >= (f.S > 256 ? 2.0 : 4.0) && takes(f, kTwoPerSm) ? kTwoPerSm : kOnePerSm;
   if (load >= 6.0 && takes(f, kNarrow)) return kNarrow;
-  if (load > (f.S <= 48 ? 1.0 : 4.0) && takes(f, kMid)) return kMid;
+  if (load > (f.S <= 44 ? 1.0 : f.S <= 48 ? 1.1 : 4.0) && takes(f, kMid)) return kMid;
   if (load >= (f.S <= 96 ? 1.5 : one.mixed && f.S > 112 ? 6.0 : 4.0) && takes(f, kTwoPerSm)) return kTwoPerSm;
   return kOnePerSm;
 }
