@@ -65,7 +65,7 @@ namespace {
 
 constexpr int NT = CBX_THREADS;  // threads per CTA (one cell at a time)
 constexpr int NW = NT / 32;
-static_assert(NT == 32 || NT == 64 || NT == 128 || NT == 256, "a cell's threads");
+static_assert(NT == 64 || NT == 128 || NT == 256, "a cell's threads");
 constexpr int kNewtonMaxIter = 4;
 constexpr int kMaxColRegs = CBX_MAX_S / 32;  // column groups per lane in the LU update
 constexpr unsigned FULL = 0xffffffffu;
@@ -76,13 +76,11 @@ __device__ __forceinline__ int tid() { return threadIdx.x; }
 
 // Barrier among the threads of a cell.
 __device__ __forceinline__ void csync() {
-  if constexpr (NT == 32) __syncwarp();
-  else __syncthreads();
+  __syncthreads();
 }
 
 __device__ __forceinline__ int csync_or(int p) {
-  if constexpr (NT == 32) return __any_sync(FULL, p);
-  else return __syncthreads_or(p);
+  return __syncthreads_or(p);
 }
 
 __device__ __forceinline__ unsigned long long globaltimer() {
@@ -467,11 +465,11 @@ __device__ __forceinline__ void crout_rows(const PivLists& P, double* M, double*
       __syncwarp();
       prep_pivot(P, M, invd, k + 1, lane);
     }
-    if (NW > 1) return;
+    return;
   }
   const int first = next_in_l ? l0 + 1 : l0;
-  const int nw = next_in_l && NW > 1 ? NW - 1 : NW;
-  const int wi = next_in_l && NW > 1 ? w - 1 : w;
+  const int nw = next_in_l ? NW - 1 : NW;
+  const int wi = next_in_l ? w - 1 : w;
   for (int e = first + wi; e < l1; e += 2 * nw) {
     const bool two = e + nw < l1;
     double* r0 = M + lrow(P, dense, k, e) * ld;
@@ -592,10 +590,10 @@ __device__ __forceinline__ void dense_first_rows(double* M, double* invd, int S,
         if (e < nu) rq[c0 + e] = e <= 1 ? xq[m] : xq[m] * inv_q;
       }
     }
-    if (NW > 1) return;
+    return;
   }
-  const int first = c0 + 2, nrow = S - first, nw = NW > 1 ? NW - 1 : 1;
-  for (int e = NW > 1 ? w - 1 : 0; e < nrow; e += 2 * nw) {
+  const int first = c0 + 2, nrow = S - first, nw = NW - 1;
+  for (int e = w - 1; e < nrow; e += 2 * nw) {
     const bool two = e + nw < nrow;
     double* r0 = M + (first + e) * ld;
     double* r1 = two ? r0 + nw * ld : r0;
@@ -748,23 +746,19 @@ __device__ __forceinline__ void urows_wait(int step, int w) {
 
 // A worker has done its first rows of this step.
 __device__ __forceinline__ void first_send(int step) {
-  if constexpr (NW > 1) {
-    if (step & 1) bar_arrive<2, NT>();
-    else bar_arrive<1, NT>();
-  }
+  if (step & 1) bar_arrive<2, NT>();
+  else bar_arrive<1, NT>();
 }
 
 __device__ __forceinline__ void first_wait(int step) {
-  if constexpr (NW > 1) {
-    if (step & 1) bar_wait<2, NT>();
-    else bar_wait<1, NT>();
-  }
+  if (step & 1) bar_wait<2, NT>();
+  else bar_wait<1, NT>();
 }
 
 // One step of the workers (every warp but warp 0).
 template <int MC>
 __device__ __forceinline__ void pair_rows(double* M, int S, int k, int step, int w, int lane) {
-  constexpr int nw = NW > 1 ? NW - 1 : 1;
+  constexpr int nw = NW - 1;
   const int ld = lead_dim(S), first = k + 4;
   const PairStep<MC> st(M, S, k, lane);
   bool sent = false;
@@ -879,8 +873,7 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
         if (step > 0) first_wait(step - 1);
         by_groups(S - k - 1, [&](auto mc) { pair_finish<mc.value>(M, invd, S, k, lane); });
         urows_send(step);
-      }
-      if (w > 0 || NW == 1) {
+      } else {
         if (step > 0) urows_wait(step - 1, w);
         by_groups(S - k - 1, [&](auto mc) { pair_rows<mc.value>(M, S, k, step, w, lane); });
       }
@@ -912,10 +905,10 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
 constexpr int LA_COLS = 8;
 
 // bulk-update worker index of warp w (of eight warps the six not on warp 0's
-// sub-partition; of one the only one), or -1
+// sub-partition, of four three, of two the second), or -1
 __device__ __forceinline__ int la_worker(int w) {
   if (NW >= 4) return (w & 3) == 0 ? -1 : (w >> 2) * 3 + (w & 3) - 1;
-  return NW == 2 ? w - 1 : 0;
+  return w - 1;
 }
 constexpr int LA_WORKERS = NW >= 4 ? (NW / 4) * 3 : 1;
 
