@@ -162,7 +162,7 @@ struct GradArgs {
 struct OrderArgs {
   int C;
   const cbx_cell_params* phi;  // [C], or null with a track
-  const double* track;         // [C][K][6] or null (its first knot counts)
+  const double* track;         // [C][K][6] or null
   int K;
   double t0, t_end;
   const double* t_end_cell;    // [C] or null
