@@ -433,9 +433,9 @@ int cbx_server_destroy(cbx_server* server);
  *   uploaded by cbx_network_create when a GPU is present); otherwise CBX_E_ARG.
  * - Limit: each CTA needs 8 * (3 R + nnz(J)) bytes of scratch (rounded up to
  *   256 B), plus, for networks whose Newton matrix does not fit in shared
- *   memory (S > 256, e.g. 500 species), the matrix itself:
- *   S * (S | 1) * 8 bytes (CBX_FP64) or * 4 bytes (CBX_MIXED). The number of
- *   CTAs launched is min(C, CTAs the device can run, CTAs that fit in the
+ *   memory (e.g. 500 species), the matrix itself: S rows of S entries rounded up
+ *   to four times an odd number, 8 bytes each (CBX_FP64) or 4 (CBX_MIXED). The
+ *   number of CTAs launched is min(C, CTAs the device runs, CTAs that fit in the
  *   16 MiB); for the 500-species / 6000-reaction network that is 7 CTAs
  *   (FP64) or 12 (CBX_MIXED) instead of one per SM, about 20x slower than
  *   cbx_solve, with the same results. Networks the solver cannot run at all

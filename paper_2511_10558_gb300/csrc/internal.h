@@ -181,12 +181,12 @@ int launch_reduce_cells(const double* gcell, int C, int R, double* out, void* st
 int launch_env_grad(const double* gcell, int C, const DevNet& n, double* g_lnzeta, double* g_lnG0, double* g_AV,
                     void* stream);
 
-// Launch plan of the solver kernel for one network and precision: matrix in
-// shared memory (gm = false) or in the CTA's global workspace (gm = true).
 // CTA shapes of the solver kernel: 256 threads and an SM to themselves (the
 // fastest a single cell gets), or several CTAs (cells) per SM for batches.
 enum CtaShape { kOnePerSm = 0, kNarrow = 1, kMid = 2, kTwoPerSm = 3 };
 
+// Launch plan of the solver kernel for one network and precision: matrix in
+// shared memory (gm = false) or in the CTA's global workspace (gm = true).
 struct SolverPlan {
   bool mixed = false, gm = false;
   size_t smem = 0;          // dynamic shared memory per CTA
@@ -196,12 +196,14 @@ struct SolverPlan {
   int sms = 0;              // of the device
   CtaShape shape = kOnePerSm;
 };
+
 // What the plan of a launch is chosen from.
 struct LaunchForms {
   int S = 0, R = 0, nseg = 0;
   size_t lean = 0;     // dynamic shared memory per CTA of the lean layout
   SolverPlan form[4];  // by CtaShape, with their occupancies
 };
+
 size_t smem_bytes(int S, int R, int nseg, bool mixed, bool gm, int piv_ints = 0);
 long long workspace_doubles(int S, int R, int nnzJ, bool mixed, bool gm);
 // The plan of a launch of C cells with at most max_ctas CTAs (0: no limit). Its

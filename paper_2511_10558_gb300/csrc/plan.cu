@@ -89,10 +89,10 @@ bool takes(const LaunchForms& f, CtaShape shape) {
 //               two        479         663   860
 // The line moves with the span, as the costliest cells' share does: 150 mixed, 912
 // cells over 1e2 and 1e6 yr, one 48 and 175, two 37 and 146; 500 mixed, 304 cells
-// over 1e4 yr, one 218, two 268. The ESDIRK's solves are more of its
-// time, which moves it too; just above one cell an SM, at 45 to 48 species, mid
-// was slower with it than one to an SM (153 cells of 48: 53 against 49 ms; 160: 41
-// against 38), so mid begins there at 1.1.
+// over 1e4 yr, one 218, two 268. The ESDIRK's solves are more of its time, which
+// moves it too; just above one cell an SM, at 45 to 48 species, mid was slower
+// with it than one to an SM (153 cells of 48: 53 against 49 ms; 160: 41 against
+// 38), so mid begins there at 1.1.
 CtaShape batch_shape(const LaunchForms& f, int C) {
   const SolverPlan& one = f.form[kOnePerSm];
   const double load = (double)C / one.sms;  // cells per SM

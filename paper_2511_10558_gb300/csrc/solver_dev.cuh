@@ -104,8 +104,9 @@ __device__ __forceinline__ int next_cell(int* counter, const int* order, int C) 
 // chunks and does what follows from the sum (the division and root, the rate
 // test, a power) alone: an FP64 instruction holds its sub-partition's pipe for
 // 64 cycles for each warp that issues it, and a division or root is a dozen of
-// them, so eight warps computing the same scalars hold it for thousands of cycles. Results go through `red`, in the half that the previous reduction
-// did not use, so that no barrier has to protect its readers.
+// them, so eight warps computing the same scalars hold it for thousands of
+// cycles. Results go through `red`, in the half that the previous reduction did
+// not use, so that no barrier has to protect its readers.
 constexpr int kChunks = 8;
 
 // Partial sums of (a v_i w_i)^2 into slot[0..7]; no barrier.
@@ -357,12 +358,13 @@ __device__ void build_matrix(const DevNet& n, const double* Jv, double c, LT* M)
 // upper triangular, in place, without pivoting, on the static fill pattern.
 // Row k of U is stored pre-scaled by 1/pivot_k, so every warp applies the
 // rank-1 update a_ij -= a_ik u_kj (rows i of L(:,k), columns j of U(k,:)) with
-// no separate scaling phase: one barrier per pivot in the sparse range. Warp 0
-// updates row k+1 first and then prepares pivot k+1 (reciprocal pivot, row
-// scaling) while the other warps work on their rows. Pivots k >= kd are
-// factored over the full ranges k+1..S-1 (entries outside the pattern are
-// exact zeros), without the per-pivot index lists, and there two pivots share
-// one barrier (PairStep).
+// no separate scaling phase. Sparse pivots take one barrier each (warp 0 updates
+// row k+1 first and then prepares pivot k+1, reciprocal and row scaling, while
+// the other warps work on their rows), or two a run where consecutive ones are
+// independent (crout_run). Pivots k >= kd are factored over the full ranges
+// k+1..S-1 (entries outside the pattern are exact zeros), without the per-pivot
+// index lists, and, once at most 128 columns remain, two a step in a pipeline of
+// warps without block barriers (PairStep).
 
 // Index lists of the sparse pivots k < kd (from the network tables, or a
 // copy of their head in shared memory).
@@ -519,8 +521,7 @@ constexpr bool kRuns = NT == 256;
 // then all rows take their updates. Two barriers a run where single pivots take
 // one each, and behind each of those waited for warp 0's reciprocal and scaling:
 // 150 species has 23 sparse pivots in runs of 10, 7, 3 and 3. 150 species, 1,216
-// cells to 1 Myr 393 -> 385 ms; 97 species ESDIRK 218 -> 215 ms; one cell of 32
-// species 13.7 -> 13.3 ms.
+// cells to 1 Myr 393 -> 385 ms; 97 species ESDIRK 218 -> 215 ms.
 __device__ void crout_run(const PivLists& P, double* M, double* invd, int k, int end, bool ready) {
   const int w = tid() >> 5, lane = tid() & 31;
   for (int m = k + (ready ? 1 : 0) + w; m < end; m += NW) prep_pivot(P, M, invd, m, lane);
@@ -858,7 +859,7 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
     }
     csync();
   }
-  if (!ready && k < S) {  // a run ended just before the pairs or the last pivot
+  if (!ready && k < S) {  // a run ended just before the pairs (or the last pivot)
     if (w == 0) prep_pivot(P, M, invd, k, lane);
     csync();
   }
@@ -892,9 +893,10 @@ __device__ void lu_crout64(const PivLists& P, double* M, double* invd) {
 }
 
 // Triangular solves with the Crout factors, blocks of 32 with look-ahead.
-// Warp w runs on the SM sub-partition w % 4, and one warp issues at most one
-// FP64 instruction per ~67 cycles, so the 32-step chain of a diagonal block
-// (warp 0, shuffles) alone leaves most of the SM's FP64 pipe idle. While warp
+// Warp w runs on the SM sub-partition w % 4, which an FP64 instruction holds for
+// 64 cycles; a step of the 32-step chain of a diagonal block (warp 0, a shuffle
+// and the FMA that needs it) takes 115, and alone leaves the other three
+// sub-partitions' FP64 pipes idle. While warp
 // 0 solves block b, the warps on the other three sub-partitions apply the
 // previous block to the rows beyond the next block (one thread per row, four
 // partial sums); after the barrier, warps 0..3 (one per sub-partition,
@@ -1754,7 +1756,7 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // Lean: the rates r and the segment sums part live in the CTA's workspace (they
 // are dead outside a right-hand side, so they take the place of the Jacobian's
 // reaction partials: nseg <= R), and f shares its storage with w, psi with tmp.
-// Two CTAs then fit an SM up to 111 species in FP64 and 152 mixed.
+// Two CTAs then fit an SM up to 111 species in FP64 and 153 mixed.
 __host__ __device__ inline size_t layout(int S, int R, int nseg, bool mixed, bool gm, unsigned char* base, Smem* s,
                                          int piv_ints = 0, bool lean = false) {
   const size_t lt = mixed ? sizeof(float) : sizeof(double);
