@@ -383,8 +383,9 @@ int cbx_tape_program(const cbx_tape* tape, int cell, int* kinds, int* qs, double
  * requests for the same network with the same options and t0 are merged into
  * one launch (up to 65,536 cells), each keeping its own t_end, so that the
  * launch's persistent CTAs back-fill across requests. Admitted launches run
- * concurrently, each with at most `max_ctas` CTAs (0 = the whole device); a
- * cell's solver state stays on chip for its whole solve. Results are bitwise
+ * concurrently, each with at most `max_ctas` CTAs (0 = the whole device), or as
+ * many SMs' worth where several CTAs share an SM (small networks); a cell's
+ * solver state stays on chip for its whole solve. Results are bitwise
  * the same whatever else is in flight or merged.
  *   mem_budget: 0 = 80 % of the device memory free at creation; otherwise a
  *               cap, itself limited to that figure.

@@ -245,17 +245,14 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (rc) return rc;
   const HostNet& h = net->host;
   const bool mixed = o.precision == CBX_MIXED;
-  auto plan_for = [&](int cells, int max_ctas) {
-    return plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, cells, max_ctas);
-  };
-  SolverPlan plan = plan_for(C, limits.max_ctas);
+  SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C, limits);
   if (plan.occupancy < 1) {
     char m[200];
     snprintf(m, sizeof m, "network (S=%d, R=%d) needs %zu B of shared memory per CTA (S <= %d); the device allows %zu",
              h.S, h.R, plan.smem, 512, device_smem_optin());
     return fail(CBX_E_TOO_LARGE, m);
   }
-  int grid = launch_grid(plan, C, limits.max_ctas);
+  int grid = launch_grid(plan, C, limits);
   cudaStream_t st = (cudaStream_t)stream;
   SolveArgs a{};
   a.net = net->dev;
@@ -294,8 +291,8 @@ static int solve_impl(cbx_network* net, const cbx_cell_params* phi, const double
   if (e == cudaErrorMemoryAllocation && (plan.shape != kOnePerSm || ordered)) {
     // no memory for several cells to an SM or for the order: the least workspace
     cudaGetLastError();
-    plan = plan_for(1, 0);
-    grid = launch_grid(plan, C, limits.max_ctas);
+    plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, 1, {});
+    grid = launch_grid(plan, C, limits);
     ordered = false;
     e = cudaMallocAsync(&ws, ws_bytes(), st);
   }

@@ -197,6 +197,14 @@ struct SolverPlan {
   CtaShape shape = kOnePerSm;
 };
 
+// What a launch may take of the device (0: no cap): the SMs' worth of CTAs, the
+// CTAs, and whether it has memory for the order of its cells.
+struct LaunchLimits {
+  int max_sms = 0;
+  int max_ctas = 0;
+  bool order = true;
+};
+
 // What the plan of a launch is chosen from.
 struct LaunchForms {
   int S = 0, R = 0, nseg = 0;
@@ -206,15 +214,15 @@ struct LaunchForms {
 
 size_t smem_bytes(int S, int R, int nseg, bool mixed, bool gm, int piv_ints = 0);
 long long workspace_doubles(int S, int R, int nnzJ, bool mixed, bool gm);
-// The plan of a launch of C cells with at most max_ctas CTAs (0: no limit). Its
-// workspace per CTA depends on neither.
-SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C, int max_ctas);
-// The same without a CUDA call at the choice: the forms, for launches of up to
-// max_ctas CTAs (0: no limit), and the plan from them.
-LaunchForms launch_forms(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int max_ctas);
-SolverPlan choose_form(const LaunchForms& f, int C, int max_ctas);
+// The plan of a launch of C cells within limits. Its workspace per CTA depends on
+// neither.
+SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C,
+                       const LaunchLimits& limits);
+// The same without a CUDA call at the choice: the forms, and the plan from them.
+LaunchForms launch_forms(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints);
+SolverPlan choose_form(const LaunchForms& f, int C, const LaunchLimits& limits);
 // The CTAs of that launch.
-int launch_grid(const SolverPlan& p, int C, int max_ctas);
+int launch_grid(const SolverPlan& p, int C, const LaunchLimits& limits);
 // Launch the solver; returns a cudaError_t value.
 int launch_solver(const SolveArgs& a, const SolverPlan& p, int grid, void* stream);
 // One translation unit per kernel instantiation (precision x matrix placement).
@@ -250,12 +258,6 @@ int launch_solve_mixed_gm_rk(const SolveArgs& a, size_t smem, int grid, void* st
 // Launch the ESDIRK solver; returns a cudaError_t value.
 int launch_solver_rk(const SolveArgs& a, const SolverPlan& p, int grid, void* stream);
 int device_sm_count();
-// What a launch may take of the device: its CTAs (0: no cap), and whether it has
-// memory for the order of its cells.
-struct LaunchLimits {
-  int max_ctas = 0;
-  bool order = true;
-};
 // cbx_solve on device buffers within limits and, optionally, with per-cell end
 // times t_end_cell [C] (device; t_end must then be their maximum).
 int solve_device(cbx_network* net, const cbx_cell_params* phi, const double* x0, int C, double t0, double t_end,

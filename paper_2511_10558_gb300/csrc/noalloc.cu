@@ -117,7 +117,7 @@ extern "C" int cbx_solve_noalloc(cbx_network* net, const cbx_cell_params* phi, c
   }
   const HostNet& h = net->host;
   const bool mixed = o.precision == CBX_MIXED;
-  const SolverPlan one = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, 1, 0);
+  const SolverPlan one = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, 1, {});
   if (one.occupancy < 1) return fail(CBX_E_TOO_LARGE, "network too large for the solver");
   const long long stride = one.ws_stride;
   const long long fit = (long long)((kScratchBytes - kCounterBytes) / (stride * sizeof(double)));
@@ -127,9 +127,10 @@ extern "C" int cbx_solve_noalloc(cbx_network* net, const cbx_cell_params* phi, c
              (long long)(stride * sizeof(double)), kScratchBytes - kCounterBytes);
     return fail(CBX_E_TOO_LARGE, m);
   }
-  const int max_ctas = (int)std::min<long long>(fit, C);
-  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C, max_ctas);
-  const int grid = launch_grid(plan, C, max_ctas);
+  LaunchLimits limits;
+  limits.max_ctas = (int)std::min<long long>(fit, C);
+  const SolverPlan plan = plan_solver(h.S, h.R, h.nseg, h.nnzJ, mixed, h.head_ints, C, limits);
+  const int grid = launch_grid(plan, C, limits);
   SolveArgs a{};
   a.net = net->dev;
   a.alpha = net->dev.alpha;

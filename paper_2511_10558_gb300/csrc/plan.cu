@@ -146,44 +146,48 @@ LaunchForms base_form(int S, int R, int nseg, int nnzJ, bool mixed, int head_int
 }
 
 template <typename Form>
-SolverPlan choose(const LaunchForms& f, int C, int max_ctas, Form form) {
-  if (max_ctas > 0 && max_ctas <= f.form[kOnePerSm].sms) return f.form[kOnePerSm];
+SolverPlan choose(const LaunchForms& f, int C, const LaunchLimits& limits, Form form) {
+  const SolverPlan& one = f.form[kOnePerSm];
+  const int ctas = limits.max_ctas;
+  if (ctas > 0 && ctas <= one.sms) return one;
+  // (Under a cap on SMs too the cells count against the whole device, which other
+  // launches share: against the capped SMs a server's requests took 8.70 s, so
+  // 8.44; small bursts 17.4 and 16.7 ms.)
   const SolverPlan p = form(batch_shape(f, C));
   // A limit that leaves less than half of the shape's CTAs: the shape for as many
   // cells as it lets run at a time (48 species, 150 CTAs: narrow 23 ms, one to an
   // SM 15; 150 species mixed, 204 of 304 CTAs: two to an SM 126, one 130).
-  return max_ctas > 0 && max_ctas < launch_grid(p, C, 0) / 2 ? form(batch_shape(f, max_ctas)) : p;
+  return ctas > 0 && ctas < std::min(C, p.occupancy * one.sms) / 2 ? form(batch_shape(f, ctas)) : p;
 }
 
 }  // namespace
 
-LaunchForms launch_forms(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int max_ctas) {
+LaunchForms launch_forms(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints) {
   LaunchForms f = base_form(S, R, nseg, nnzJ, mixed, head_ints);
-  const SolverPlan& one = f.form[kOnePerSm];
-  if (one.occupancy < 1) return f;
-  for (CtaShape shape : {kNarrow, kMid, kTwoPerSm}) {
-    if ((max_ctas == 0 || max_ctas > one.sms) && takes(f, shape)) query_form(f, shape);
-    else f.form[shape] = one;
-  }
+  if (f.form[kOnePerSm].occupancy < 1) return f;
+  for (CtaShape shape : {kNarrow, kMid, kTwoPerSm})
+    if (takes(f, shape)) query_form(f, shape);
   return f;
 }
 
-SolverPlan choose_form(const LaunchForms& f, int C, int max_ctas) {
-  return choose(f, C, max_ctas, [&](CtaShape s) { return f.form[s]; });
+SolverPlan choose_form(const LaunchForms& f, int C, const LaunchLimits& limits) {
+  return choose(f, C, limits, [&](CtaShape s) { return f.form[s]; });
 }
 
-SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C, int max_ctas) {
+SolverPlan plan_solver(int S, int R, int nseg, int nnzJ, bool mixed, int head_ints, int C,
+                       const LaunchLimits& limits) {
   LaunchForms f = base_form(S, R, nseg, nnzJ, mixed, head_ints);
   if (f.form[kOnePerSm].occupancy < 1) return f.form[kOnePerSm];
-  return choose(f, C, max_ctas, [&](CtaShape s) {
+  return choose(f, C, limits, [&](CtaShape s) {
     if (s != kOnePerSm) query_form(f, s);
     return f.form[s];
   });
 }
 
-int launch_grid(const SolverPlan& p, int C, int max_ctas) {
-  const int grid = std::min(C, p.occupancy * p.sms);
-  return max_ctas > 0 ? std::min(grid, max_ctas) : grid;
+int launch_grid(const SolverPlan& p, int C, const LaunchLimits& limits) {
+  const int sms = limits.max_sms > 0 ? std::min(limits.max_sms, p.sms) : p.sms;
+  const int grid = std::min(C, p.occupancy * sms);
+  return limits.max_ctas > 0 ? std::min(grid, limits.max_ctas) : grid;
 }
 
 int launch_solver(const SolveArgs& a0, const SolverPlan& p, int grid, void* stream) {

@@ -8,8 +8,8 @@
 // the launch's persistent CTAs back-fill across requests; a cell's solver
 // state stays on chip for its whole solve. Requests that arrive while others
 // run are admitted into the freed streams and memory, and their kernels run
-// concurrently with the running ones; each launch uses at most `max_ctas` CTAs
-// so that several launches, of any network size, share the SMs.
+// concurrently with the running ones; each launch uses at most `max_ctas` SMs'
+// worth of CTAs so that several launches, of any network size, share the SMs.
 //
 // Per launch: device buffers (inputs, outputs, per-cell end times, solver
 // workspace), the H2D copies of every merged request (strided copies into the
@@ -115,7 +115,7 @@ namespace {
 // so only outside the server's lock.
 void size_request(ServerRequest* r, int max_ctas) {
   const HostNet& h = r->net->host;
-  r->forms = launch_forms(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints, max_ctas);
+  r->forms = launch_forms(h.S, h.R, h.nseg, h.nnzJ, r->opt.precision == CBX_MIXED, h.head_ints);
   const SolverPlan& one = r->forms.form[kOnePerSm];
   r->cell_bytes = sizeof(cbx_cell_params) + 2 * h.S * sizeof(double) + sizeof(double) + sizeof(int);
   r->cta_bytes = (size_t)one.ws_stride * sizeof(double);
@@ -128,7 +128,7 @@ void size_request(ServerRequest* r, int max_ctas) {
 // end times, status, workspace, order of the cells (pure arithmetic: safe under
 // the lock).
 size_t launch_bytes(const ServerRequest* r, int C, const LaunchLimits& limits) {
-  const int grid = std::max(1, launch_grid(choose_form(r->forms, C, limits.max_ctas), C, limits.max_ctas));
+  const int grid = std::max(1, launch_grid(choose_form(r->forms, C, limits), C, limits));
   return (size_t)C * r->cell_bytes + grid * r->cta_bytes + (limits.order && C > grid ? (size_t)C * sizeof(int) : 0) +
          8192;
 }
@@ -259,7 +259,7 @@ ServerLaunch* next_launch(cbx_server* s) {
   s->queue.swap(rest);
   size_t taken = s->in_use + L->bytes;
   for (ServerRequest* r : s->queue) taken += launch_bytes(r, r->C, r->least);
-  const LaunchLimits full{s->max_ctas, true};
+  const LaunchLimits full{s->max_ctas, 0, true};
   const size_t bytes = launch_bytes(head, L->C, full), extra = bytes - L->bytes;
   const size_t left = taken <= s->budget ? s->budget - taken : 0;
   const size_t streams = std::count(s->busy.begin(), s->busy.end(), 0) - 1;  // free beside this launch's

@@ -1,7 +1,7 @@
 """What a server's limits mean, whatever shape its launches take (GPU).
 
-max_ctas is the most CTAs of a launch, for small networks too (several of whose
-CTAs could share an SM), and may be as large as an int.
+max_ctas is the most CTAs of a launch, or as many SMs' worth where several CTAs
+share an SM (up to eight, of small networks), and may be as large as an int.
 
 Reservations are checked through the server's peak: inputs, outputs and end
 times of the cells, a workspace per CTA, 8 KB. Results are bitwise those of
@@ -40,7 +40,7 @@ def _check(N, phi, x0, t_end, opt, out):
 
 @pytest.mark.parametrize("prec", [carbox.CBX_FP64, carbox.CBX_MIXED])
 @pytest.mark.parametrize("max_ctas", [1, 8, 76, 200])
-def test_max_ctas_is_a_number_of_ctas(net32, prec, max_ctas):
+def test_max_ctas_is_a_share_of_the_device(net32, prec, max_ctas):
     N = carbox.Network.from_synth(net32)
     C, opt = 400, carbox.options(precision=prec)
     phi, x0 = _request(net32, C, 1)
@@ -48,7 +48,7 @@ def test_max_ctas_is_a_number_of_ctas(net32, prec, max_ctas):
     out = srv.wait(srv.submit(N, phi, x0, 0.0, 10.0 * YR, opt))
     peak = srv.stats()["peak_bytes"]
     srv.close()
-    assert peak <= _bytes(N, C, max_ctas) + 4 * C  # and the order of the cells
+    assert peak <= _bytes(N, C, 8 * max_ctas) + 4 * C  # and the order of the cells
     _check(N, phi, x0, 10.0 * YR, opt, out)
 
 
