@@ -221,9 +221,9 @@ void launch(cbx_server* s, ServerLaunch* L) {
 // requests of the same kind that fit with it. What fits is judged by the least
 // that a launch takes; a launch gets the plan of its size (more CTAs of small
 // networks, the cells' order) where that keeps no other waiting: it costs at
-// most an eighth of the memory that the queued requests leave, and as many
-// launches of this size fit beside it as without. Returns null when nothing
-// fits.
+// most an eighth of the memory that the queued requests with a stream to run on
+// leave, and as many launches of this size fit beside it as without. Returns
+// null when nothing fits.
 ServerLaunch* next_launch(cbx_server* s) {
   auto fits = [&](size_t bytes) { return s->in_use + bytes <= s->budget || s->in_use == 0; };
   ServerRequest* head = nullptr;
@@ -257,12 +257,13 @@ ServerLaunch* next_launch(cbx_server* s) {
   for (ServerRequest* r : s->queue)
     if (std::find(L->reqs.begin(), L->reqs.end(), r) == L->reqs.end()) rest.push_back(r);
   s->queue.swap(rest);
+  const size_t streams = std::count(s->busy.begin(), s->busy.end(), 0) - 1;  // free beside this launch's
   size_t taken = s->in_use + L->bytes;
-  for (ServerRequest* r : s->queue) taken += launch_bytes(r, r->C, r->least);
+  for (size_t k = 0; k < std::min(streams, s->queue.size()); ++k)
+    taken += launch_bytes(s->queue[k], s->queue[k]->C, s->queue[k]->least);
   const LaunchLimits full{s->max_ctas, 0, true};
   const size_t bytes = launch_bytes(head, L->C, full), extra = bytes - L->bytes;
   const size_t left = taken <= s->budget ? s->budget - taken : 0;
-  const size_t streams = std::count(s->busy.begin(), s->busy.end(), 0) - 1;  // free beside this launch's
   auto beside = [&](size_t room) { return std::min(streams, room / L->bytes); };
   if (extra <= left / 8 && beside(left - extra) == beside(left)) {
     L->limits = full;

@@ -76,6 +76,27 @@ def test_room_for_several_cells_on_an_sm_is_used(net32):
     _check(N, phi, x0, YR, opt, out)
 
 
+def test_a_long_queue_leaves_the_shapes(net32, net150):
+    # one stream, held by a long cell; behind it a batch that runs several cells to an SM, and forty requests
+    # (one cell to an SM whatever they are given) that exceed the budget together but wait for the stream
+    net61 = synth.make_network(61, 480)
+    N32, N61, N150 = (carbox.Network.from_synth(n) for n in (net32, net61, net150))
+    opt = carbox.options()
+    phi, x0 = _request(net32, 2000, 6)
+    one = _bytes(N61, _sms(), _sms())
+    budget = 34 * one
+    srv = carbox.Server(mem_budget=budget, n_streams=1, max_ctas=0)
+    ids = [srv.submit(N150, *_request(net150, 1, 7), 0.0, 1e7 * YR, opt), srv.submit(N32, phi, x0, 0.0, YR, opt)]
+    many = _request(net61, _sms(), 8)
+    ids += [srv.submit(N61, *many, float(k), YR, opt) for k in range(40)]  # not merged: different start times
+    outs = [srv.wait(i) for i in ids]
+    peak = srv.stats()["peak_bytes"]
+    srv.close()
+    assert _bytes(N32, 2000, 4 * _sms()) <= peak <= budget
+    _check(N32, phi, x0, YR, opt, outs[1])
+    assert all(np.all(st == carbox.CBX_CELL_OK) for _, st, _ in outs)
+
+
 def test_requests_run_side_by_side_where_their_least_fits(net150):
     N = carbox.Network.from_synth(net150)
     opt = carbox.options(precision=carbox.CBX_MIXED)
